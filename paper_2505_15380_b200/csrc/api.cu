@@ -30,6 +30,8 @@ int cuda_fail(cudaError_t e, const char* what) {
 inline size_t align_up(size_t v, size_t a = 256) { return (v + a - 1) / a * a; }
 
 constexpr size_t PREFILL_ROWS = 64;  // least rows a bf16 streams object can run in one forward
+constexpr int TC_CHECK_ROWS = 512;  // rows of the stand-alone projection call
+constexpr size_t SPLIT_KEY_ROWS = TC_MAX_ROWS;  // prefill chunks of up to this many rows may split their attention's keys
 // Streams with room for this many tokens run the persistent kernel's key-split variant: from a
 // few hundred keys on, ten CTAs sharing a head's keys and meeting once costs less than each of
 // them walking all keys (0.8 us per 128 keys and layer against ~1.5 us for the exchange).
@@ -143,11 +145,11 @@ struct WsPlan {
   size_t h, qkv, qrot, rope_cs, part, logits, row_stats, xn, attn_out, act;
   size_t st_tokens, st_k, st_y, st_probs, st_uni;
   size_t hfix, flags, epoch_base, xa, xb, xd, xq, ssq_a, ssq_b;
-  size_t tc_xa, tc_xattn, tc_xact, tc_part;
+  size_t tc_rowmap, tc_tiles, tc_xa, tc_xattn, tc_xact, tc_part;
   size_t attn_part, attn_cnt;
   size_t page_table, pages_used, free_stack, free_top;
   size_t total;
-  int max_rows, nsplit_max;
+  int max_rows, nsplit_max, tc_rows, tc_part_rows;
 };
 
 WsPlan plan_ws(const ssd_model_config& c, int B, int max_gamma, int cap, int n_pages = 0, int max_pages = 0) {
@@ -159,19 +161,30 @@ WsPlan plan_ws(const ssd_model_config& c, int B, int max_gamma, int cap, int n_p
   // bf16 models: room for prefill chunks large enough for the tensor-core forward
   if (c.weight_dtype == 1 && M < PREFILL_ROWS) M = PREFILL_ROWS;
   p.max_rows = (int)M;
+  // rows of a tensor-core forward: a prefill takes its prompts in chunks as large as the
+  // kernels allow (64-row chunks ran the same launches 32 times as often), no more than the cache holds
+  size_t MT = 0, MP = M;
+  if (c.weight_dtype == 1 && M <= TC_MAX_ROWS) {
+    MT = std::min((size_t)TC_MAX_ROWS, align_up((size_t)B * cap, 64));
+    if (MT < M) MT = M;
+    MP = std::max(M, std::min(MT, SPLIT_KEY_ROWS));
+  }
+  p.tc_rows = (int)MT;
+  p.tc_part_rows = (int)MP;
+  const size_t MX = std::max(M, MT);
   p.nsplit_max = (cap + ATTN_CHUNK - 1) / ATTN_CHUNK;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes); return o; };
   p.len = take(B * 4);
   p.pending = take(B * 4);
   p.status = take(4);
   p.counters = take(B * 4);
-  p.row_ids = take(M * 4);
+  p.row_ids = take(MX * 4);
   p.accept_flags = take(M * 4);
-  p.h = take(M * d * 4);
+  p.h = take(MX * d * 4);
   p.qkv = take(M * (qd + 2 * kvd) * 4);
-  p.qrot = take(M * qd * 4);
-  p.rope_cs = take(M * c.head_dim * 4);
-  p.part = take(M * c.n_q_heads * (size_t)p.nsplit_max * (c.head_dim + 2) * 4);
+  p.qrot = take(MX * qd * 4);
+  p.rope_cs = take(MX * c.head_dim * 4);
+  p.part = take(MP * c.n_q_heads * (size_t)p.nsplit_max * (c.head_dim + 2) * 4);
   p.logits = take(M * V * 4);
   p.row_stats = take(M * 8 * 4);  // eight statistics words per row (sampler.cu)
   p.xn = take(M * d * 4);
@@ -207,14 +220,18 @@ WsPlan plan_ws(const ssd_model_config& c, int B, int max_gamma, int cap, int n_p
     p.free_stack = take((size_t)n_pages * 4);
     p.free_top = take(4);
   }
-  p.tc_xa = p.tc_xattn = p.tc_xact = p.tc_part = 0;
-  if (c.weight_dtype == 1 && M > FAST_MAX_T && M <= TC_MAX_ROWS) {
-    const int Mpad = tc_round16((int)M), n_sm = fast_cta_count();
+  p.tc_xa = p.tc_xattn = p.tc_xact = p.tc_part = p.tc_rowmap = p.tc_tiles = 0;
+  if (MT > FAST_MAX_T) {
+    p.tc_rowmap = take(MT * sizeof(int2));
+    p.tc_tiles = take((MT + PREFILL_SEGS) * sizeof(int4));
+    const int Mpad = tc_round16((int)MT), Mdec = tc_round16((int)M), n_sm = fast_cta_count();
     // the row chunks of an operand depend on the rows of the forward: room for the largest
     size_t rows_max = 0;
     for (int mp = 16; mp <= Mpad; mp += 16) {
       const TcChunks ch = tc_chunks(mp);
       rows_max = std::max(rows_max, (size_t)ch.n * ch.rows);
+      const TcChunks pc = tc_prefill_chunks(mp);
+      rows_max = std::max(rows_max, (size_t)pc.n * pc.rows);
     }
     p.tc_xa = take((size_t)((d + 15) / 16) * rows_max * 64);
     p.tc_xattn = take((size_t)((qd + 15) / 16) * rows_max * 64);
@@ -224,8 +241,10 @@ WsPlan plan_ws(const ssd_model_config& c, int B, int max_gamma, int cap, int n_p
     for (int i = 0; i < 3; ++i) {
       const size_t tiles = (rows[i] + TC_TILE_ROWS - 1) / TC_TILE_ROWS;
       for (int mp = 16; mp <= Mpad; mp += 16) {  // the K split depends on the rows of the forward
-        const size_t b = (size_t)tc_ksplit(rows[i], ks[i], mp, n_sm) * mp * tiles * TC_TILE_ROWS * 4;
-        part = b > part ? b : part;
+        const size_t row_bytes = (size_t)mp * tiles * TC_TILE_ROWS * 4;
+        const int nsl = tc_ksplit(rows[i], ks[i], TC_PREFILL_CHUNK, n_sm);
+        part = std::max(part, tc_prefill_groups(rows[i], mp, nsl, n_sm) > 1 ? nsl * row_bytes : row_bytes);
+        if (mp <= Mdec) part = std::max(part, tc_ksplit(rows[i], ks[i], mp, n_sm) * row_bytes);
       }
     }
     p.tc_part = take(part);
@@ -250,7 +269,7 @@ bool same_shape(const ssd_model_config& a, const ssd_model_config& b) {
 // rows' K/V at len + r; when logits_out is non-null also runs the final norm and the LM head.
 // The persistent kernel covers forwards of at most FAST_MAX_T rows over a bf16 model.
 bool use_fast(const ssd_model* m, const ssd_streams* s, RowMap rm) {
-  return m->fast.enabled && s->path == 0 && !s->paged && rm.nb * rm.R <= FAST_MAX_T;
+  return m->fast.enabled && s->path == 0 && !s->paged && !rm.rows && rm.nb * rm.R <= FAST_MAX_T;
 }
 
 int forward_fast(const ssd_model* m, ssd_streams* s, RowMap rm, const int32_t* row_ids,
@@ -322,65 +341,86 @@ int forward_fast(const ssd_model* m, ssd_streams* s, RowMap rm, const int32_t* r
 // Forwards of more than FAST_MAX_T rows over a bf16 model: projections on the tcgen05 tensor cores
 // (each weight byte read once), attention on the warp-level tensor-core instruction.
 bool use_tc(const ssd_model* m, const ssd_streams* s, RowMap rm) {
-  const int M = rm.nb * rm.R;
+  const int M = row_count(rm);
   if (s->paged) return true;  // the paged cache exists on this path only (sizes checked at creation)
-  return m->tc.enabled && s->path == 0 && s->tc_part && M > FAST_MAX_T && M <= TC_MAX_ROWS && M <= s->max_rows;
+  return m->tc.enabled && s->path == 0 && s->tc_part && M > FAST_MAX_T && M <= s->tc_rows;
 }
 
-int forward_tc(const ssd_model* m, ssd_streams* s, RowMap rm, float* logits_out, cudaStream_t st) {
+int forward_tc(const ssd_model* m, ssd_streams* s, RowMap rm, float* logits_out, cudaStream_t st,
+               const PrefillSegs* segs = nullptr) {
   const ssd_model_config& c = m->cfg;
-  const int M = rm.nb * rm.R, Mpad = tc_round16(M), d = c.d_model;
+  const int M = row_count(rm), Mpad = tc_round16(M), d = c.d_model;
   const int qd = c.n_q_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim, F = c.d_ffn, nq = qd + 2 * kvd;
   const int n_sm = m->tc.n_sm;
   auto ld_of = [](int rows) { return (rows + TC_TILE_ROWS - 1) / TC_TILE_ROWS * TC_TILE_ROWS; };
-  const int ks_qkv = tc_ksplit(nq, d, M, n_sm), ks_o = tc_ksplit(d, qd, M, n_sm), ks_d = tc_ksplit(d, F, M, n_sm);
+  const int Mks = rm.rows ? TC_PREFILL_CHUNK : M;
+  const int ks_qkv = tc_ksplit(nq, d, Mks, n_sm), ks_o = tc_ksplit(d, qd, Mks, n_sm), ks_d = tc_ksplit(d, F, Mks, n_sm);
   // key splits of the attention: whole 64-key tiles, and no more CTAs in all than the SMs hold
   // at once (a second, partly filled wave would cost as much as the first)
   const int G = c.n_q_heads / c.n_kv_heads, rowgroups = (G * rm.R + 63) / 64;
+  // a prefill's rows are summed as a forward of max_rows rows would sum them, whatever the chunk holds
+  const bool seg = rm.rows != nullptr;
+  const int Mc = seg ? tc_prefill_chunks(M).rows : tc_chunks(M).rows;
   long long want = ((long long)tc_attention_ctas_per_sm(c.head_dim) * n_sm) /
-                   ((long long)rm.nb * c.n_kv_heads * rowgroups);  // splits that still fit one wave
+                   (seg ? (long long)c.n_kv_heads * ((G * s->max_rows + 63) / 64)
+                        : (long long)rm.nb * c.n_kv_heads * rowgroups);  // splits that still fit one wave
   if (want < 1) want = 1;
   long long kps = ((s->cap + want - 1) / want + 63) / 64 * 64;
   if (kps < 64) kps = 64;
-  while ((s->cap + kps - 1) / kps > 128) kps += 64;  // the merge kernel's table of splits
+  while (want > 1 && (s->cap + kps - 1) / kps > 128) kps += 64;  // the merge kernel's table of splits
   const int nsplit = (int)((s->cap + kps - 1) / kps);
-  if (M > s->max_rows || M > TC_MAX_ROWS) return SSD_ERR_BAD_PARAM;
-  if (s->paged)  // every stream of this forward owns pages for the rows it is about to append
+  if (M > s->tc_rows) return SSD_ERR_BAD_PARAM;
+  if (s->paged && segs)
+    launch_page_ensure_segs(s->len, *segs, s->page_table, s->pages_used, s->free_stack, s->free_top, s->max_pages,
+                            s->status, st);
+  else if (s->paged)  // every stream of this forward owns pages for the rows it is about to append
     launch_page_ensure(s->len, rm, s->page_table, s->pages_used, s->free_stack, s->free_top, s->max_pages,
                        s->status, st);
   launch_embed(1, m->embed, c.vocab_out + c.vocab_text, d, s->row_ids, M, s->h, s->status, st);
   launch_rope_table(s->len, rm, m->inv_freq, c.head_dim / 2, s->rope_cs, st);
+  // prefill: whether a projection's slices are added within its CTAs, or written out one by one
+  const bool in_qkv = seg && tc_prefill_groups(nq, M, ks_qkv, n_sm) == 1, in_o = seg && tc_prefill_groups(d, M, ks_o, n_sm) == 1,
+             in_d = seg && tc_prefill_groups(d, M, ks_d, n_sm) == 1;
+  auto lay = [&](int K) { return seg ? tc_act_lay_parts(Mc, K) : tc_act_lay(Mc, K); };
+  auto gemm = [&](const TcGemm& q, bool in_cta, int epi, const void* bias, float* out) {
+    if (!seg) return launch_tc_gemm(q, st);
+    return launch_tc_prefill_gemm(q, in_cta || epi == PF_EPI_SWIGLU ? epi : PF_EPI_PARTIAL, (const bf16*)bias,
+                                  in_cta ? out : q.part, n_sm, st, lay(q.n_rows / 2));
+  };
   const float* part = nullptr;
   int nsp = 0, ldp = 0;
   TcGemm g{};
   g.M = M;
+  g.mc = seg ? Mc : 0;
   g.status = s->status;
   for (int l = 0; l < c.n_layers; ++l) {
     const LayerW& w = m->layers[l];
     const ssd_tc_layer& t = m->tc.layers[l];
     bf16* kv_layer = (bf16*)(s->kv + (size_t)l * s->kv_layer_elems * s->el);
-    launch_tc_norm_pack(s->h, part, nsp, ldp, M, d, (const bf16*)w.norm1, c.rms_eps, s->tc_xa, st);
+    launch_tc_norm_pack(s->h, part, nsp, ldp, M, lay(d), d, (const bf16*)w.norm1, c.rms_eps, s->tc_xa, st);
     g.w = t.w_qkv; g.a = s->tc_xa; g.n_rows = nq; g.K = d; g.ksplit = ks_qkv; g.epi = TC_EPI_PARTIAL; g.part = s->tc_part;
-    SSD_CUDA(launch_tc_gemm(g, st));
-    launch_tc_qkv_post(s->tc_part, ks_qkv, ld_of(nq), Mpad, (const bf16*)w.b_qkv, s->rope_cs, s->qrot, kv_layer,
+    SSD_CUDA(gemm(g, in_qkv, PF_EPI_BIAS, w.b_qkv, s->tc_part));
+    launch_tc_qkv_post(s->tc_part, in_qkv ? 1 : ks_qkv, in_qkv ? nq : ld_of(nq), Mpad,
+                       in_qkv ? nullptr : (const bf16*)w.b_qkv, s->rope_cs, s->qrot, kv_layer,
                        s->len, rm, s->cap, c.n_q_heads, c.n_kv_heads, c.head_dim, s->page_table, s->max_pages,
                        s->status, st);
+    if (!logits_out && l + 1 == c.n_layers) break;  // only the cache is wanted: nothing reads what follows
     SSD_CUDA(launch_tc_attention(s->qrot, kv_layer, s->len, rm, s->cap, c.n_q_heads, c.n_kv_heads, c.head_dim,
-                                 s->part, nsplit, (int)kps, s->tc_xattn, Mpad, s->page_table, s->max_pages, s->attn_kernel,
+                                 s->part, nsplit, (int)kps, s->tc_xattn, lay(qd), s->page_table, s->max_pages, s->attn_kernel,
                                  s->status, st));
     g.w = t.w_o; g.a = s->tc_xattn; g.n_rows = d; g.K = qd; g.ksplit = ks_o;
-    SSD_CUDA(launch_tc_gemm(g, st));
-    launch_tc_norm_pack(s->h, s->tc_part, ks_o, ld_of(d), M, d, (const bf16*)w.norm2, c.rms_eps, s->tc_xa, st);
+    SSD_CUDA(gemm(g, in_o, PF_EPI_RESIDUAL, nullptr, s->h));
+    launch_tc_norm_pack(s->h, in_o ? nullptr : s->tc_part, ks_o, ld_of(d), M, lay(d), d, (const bf16*)w.norm2, c.rms_eps, s->tc_xa, st);
     g.w = t.w_gu; g.a = s->tc_xa; g.n_rows = 2 * F; g.K = d; g.ksplit = 1; g.epi = TC_EPI_SWIGLU; g.act_out = s->tc_xact;
-    SSD_CUDA(launch_tc_gemm(g, st));
+    SSD_CUDA(gemm(g, false, PF_EPI_SWIGLU, nullptr, nullptr));
     g.w = t.w_d; g.a = s->tc_xact; g.n_rows = d; g.K = F; g.ksplit = ks_d; g.epi = TC_EPI_PARTIAL;
-    SSD_CUDA(launch_tc_gemm(g, st));
-    part = s->tc_part;
+    SSD_CUDA(gemm(g, in_d, PF_EPI_RESIDUAL, nullptr, s->h));
+    part = in_d ? nullptr : s->tc_part;
     nsp = ks_d;
     ldp = ld_of(d);
   }
   if (logits_out) {
-    launch_tc_norm_pack(s->h, part, nsp, ldp, M, d, (const bf16*)m->norm_f, c.rms_eps, s->tc_xa, st);
+    launch_tc_norm_pack(s->h, part, nsp, ldp, M, lay(d), d, (const bf16*)m->norm_f, c.rms_eps, s->tc_xa, st);
     g.w = m->tc.head; g.a = s->tc_xa; g.n_rows = c.vocab_out; g.K = d; g.ksplit = 1; g.epi = TC_EPI_STORE;
     g.out = logits_out; g.ldo = c.vocab_out;
     SSD_CUDA(launch_tc_gemm(g, st));
@@ -421,6 +461,65 @@ int forward(const ssd_model* m, ssd_streams* s, RowMap rm, float* logits_out, cu
     launch_rmsnorm(dt, s->h, m->norm_f, s->xn, M, d, c.rms_eps, st);
     SSD_CUDA(launch_gemm_simt(dt, EPI_STORE_F32, s->xn, d, m->head, nullptr, logits_out,
                               c.vocab_out, M, c.vocab_out, d, st));
+  }
+  SSD_CUDA(cudaGetLastError());
+  return SSD_OK;
+}
+
+// Prefill on the tensor-core path: the prompts' rows, all streams one after the other, are cut into
+// equal chunks of at most tc_rows rows; a chunk is one forward whose rows may belong to several
+// streams (causal within each).  A last chunk of few rows of one stream is the persistent kernel's.
+int prefill_tc(ssd_model* m, ssd_streams* s, const int32_t* ids, const int32_t* off, cudaStream_t st) {
+  const int G = m->cfg.n_q_heads / m->cfg.n_kv_heads;
+  long long left = 0;
+  for (int b = 0; b < s->B; ++b) left += std::max(off[b + 1] - off[b] - 1, 0);
+  const long long n_chunks = std::max<long long>((left + s->tc_rows - 1) / s->tc_rows, 1);
+  const int target = std::min((int)align_up((size_t)((left + n_chunks - 1) / n_chunks), 16), s->tc_rows);
+  int b = 0, done = 0;  // next stream, rows of it already taken
+  while (b < s->B) {
+    PrefillSegs P{};
+    P.tile_rows = 64 / G;
+    while (b < s->B && P.n < PREFILL_SEGS) {
+      const int n = off[b + 1] - off[b];
+      if (n == 0) {  // takes no part
+        ++b;
+        continue;
+      }
+      const int count = std::min(n - 1 - done, target - P.n_rows);
+      if (count == 0 && done < n - 1) break;  // the chunk is full
+      const bool ends = done + count == n - 1;
+      P.s[P.n].stream = b;
+      P.s[P.n].src = off[b] + done;
+      P.s[P.n].count = count;
+      P.s[P.n].m0 = P.n_rows;
+      P.s[P.n].tile0 = P.n_tiles;
+      P.s[P.n].pend_src = ends ? off[b] + n - 1 : -1;
+      ++P.n;
+      P.n_rows += count;
+      P.n_tiles += (count + P.tile_rows - 1) / P.tile_rows;
+      done = ends ? 0 : done + count;
+      if (ends) ++b;
+      else break;
+    }
+    if (P.n == 0) break;
+    if (P.n_rows > 0) {
+      const RowMap one{P.s[0].stream, 1, P.n_rows};
+      int rc;
+      if (P.n == 1 && use_fast(m, s, one)) {
+        SSD_CUDA(cudaMemcpyAsync(s->row_ids, ids + P.s[0].src, (size_t)P.n_rows * 4, cudaMemcpyDeviceToDevice, st));
+        rc = forward(m, s, one, nullptr, st);
+      } else {
+        RowMap rm{0, 0, 1};
+        rm.rows = s->tc_rowmap;
+        rm.tiles = s->tc_tiles;
+        rm.n_rows = P.n_rows;
+        rm.n_tiles = P.n_tiles;
+        launch_prefill_stage(P, ids, s->row_ids, s->tc_rowmap, s->tc_tiles, st);
+        rc = forward_tc(m, s, rm, nullptr, st, &P);
+      }
+      if (rc != SSD_OK) return rc;
+    }
+    launch_prefill_advance(P, ids, s->len, s->pending, st);
   }
   SSD_CUDA(cudaGetLastError());
   return SSD_OK;
@@ -780,6 +879,8 @@ int streams_create_impl(const ssd_model* m, int32_t batch, int32_t capacity_toke
   s->max_gamma = max_gamma;
   s->max_rows = p.max_rows;
   s->nsplit_max = p.nsplit_max;
+  s->tc_rows = p.tc_rows;
+  s->tc_part_rows = p.tc_part_rows;
   s->kv = (char*)dev_kv;
   s->kv_layer_elems = paged ? (size_t)n_pages * 2 * c.n_kv_heads * (size_t)TC_PAGE_TOKENS * c.head_dim
                             : (size_t)batch * 2 * c.n_kv_heads * (size_t)capacity_tokens * c.head_dim;
@@ -822,6 +923,8 @@ int streams_create_impl(const ssd_model* m, int32_t batch, int32_t capacity_toke
   s->attn_part = p.attn_part ? (float*)(W + p.attn_part) : nullptr;
   s->attn_cnt = p.attn_part ? (uint32_t*)(W + p.attn_cnt) : nullptr;
   s->key_split = capacity_tokens >= KEYSPLIT_MIN_CAPACITY ? 1 : 0;
+  s->tc_rowmap = p.tc_part ? (int2*)(W + p.tc_rowmap) : nullptr;
+  s->tc_tiles = p.tc_part ? (int4*)(W + p.tc_tiles) : nullptr;
   s->tc_xa = p.tc_part ? (uint8_t*)(W + p.tc_xa) : nullptr;
   s->tc_xattn = p.tc_part ? (uint8_t*)(W + p.tc_xattn) : nullptr;
   s->tc_xact = p.tc_part ? (uint8_t*)(W + p.tc_xact) : nullptr;
@@ -979,11 +1082,9 @@ int ssd_prefill(ssd_model* m, ssd_streams* s, const int32_t* dev_ids, const int3
     if (n - 1 > s->cap) return SSD_ERR_KV_OVERFLOW;
   }
   cudaStream_t st = (cudaStream_t)stream;
-  // rows per forward: as many as the workspace holds when the tensor-core forward can take them
-  // (one stream at a time, the chunk's rows causal among themselves), else a verify step's worth
-  int chunk = s->max_gamma + 1;
-  if (m->tc.enabled && s->path == 0 && s->tc_part && s->max_rows > FAST_MAX_T)
-    chunk = s->max_rows < TC_MAX_ROWS ? s->max_rows : TC_MAX_ROWS;
+  // generic kernels: one stream at a time, a verify step's worth of rows per forward
+  if (m->tc.enabled && s->path == 0 && s->tc_part) return prefill_tc(m, s, dev_ids, host_offsets, st);
+  const int chunk = s->max_gamma + 1;
   for (int b = 0; b < s->B; ++b) {
     const int32_t* ids = dev_ids + host_offsets[b];
     int n = host_offsets[b + 1] - host_offsets[b];
@@ -1182,7 +1283,7 @@ int ssd_last_status(ssd_streams* s, int32_t* status, void* stream) {
 }
 
 size_t ssd_tc_gemm_scratch_bytes(int32_t M, int32_t n_rows, int32_t K) {
-  if (M < 1 || M > TC_MAX_ROWS || n_rows < 1 || K < 8 || (K & 7)) return 0;
+  if (M < 1 || M > TC_CHECK_ROWS || n_rows < 1 || K < 8 || (K & 7)) return 0;
   return align_up(tc_weight_bytes(n_rows, K)) + align_up(tc_act_bytes(tc_round16(M), K));
 }
 

@@ -63,9 +63,27 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 }
 
 // Which rows a forward pass covers: streams b0..b0+nb-1, R rows each; row m = bi*R + r sits at
-// position len[b0+bi] + r of its stream.
+// position len[b0+bi] + r of its stream.  A prefill chunk instead lists its rows (several streams,
+// each with its own number of rows): `rows[m]` = (stream, r), and the attention's work items
+// `tiles` = (stream, first row m, its r, rows) of at most tile_rows rows of one stream.
 struct RowMap {
   int b0, nb, R;
+  const int2* rows = nullptr;
+  const int4* tiles = nullptr;
+  int n_rows = 0, n_tiles = 0;
+};
+inline int row_count(const RowMap& rm) { return rm.rows ? rm.n_rows : rm.nb * rm.R; }
+__device__ __forceinline__ int2 row_at(const RowMap& rm, int m) {  // (stream, r) of row m
+  return rm.rows ? rm.rows[m] : make_int2(rm.b0 + m / rm.R, m % rm.R);
+}
+
+// The streams of a prefill chunk: `count` consecutive ids of `stream` from ids[src] on become rows
+// m0.. of the forward (attention tiles tile0..); pend_src >= 0: the stream's prompt ends with this
+// chunk and ids[pend_src] is its pending token.
+constexpr int PREFILL_SEGS = 32;
+struct PrefillSegs {
+  int n, n_rows, n_tiles, tile_rows;
+  struct { int stream, src, count, m0, tile0, pend_src; } s[PREFILL_SEGS];
 };
 
 struct LayerW {
@@ -114,6 +132,7 @@ struct ssd_streams {
   ssd_model_config cfg;  // shape the cache was laid out for
   int el;
   int B, cap, max_gamma, max_rows, nsplit_max;
+  int tc_rows, tc_part_rows;  // most rows of a tensor-core forward, and of one whose attention splits the keys
   char* kv;
   size_t kv_layer_elems;  // elements per layer: B * 2 * Hkv * cap * hd
   char* ws;
@@ -139,6 +158,8 @@ struct ssd_streams {
   int32_t *page_table, *pages_used, *free_stack, *free_top;
   // batched tensor-core forward: packed operands (inputs of QKV / gate-up / head, of O, of down)
   // and the partial sums of the K-split projections
+  int2* tc_rowmap;  // prefill chunks: (stream, r) of every row, and the attention's tiles
+  int4* tc_tiles;
   uint8_t *tc_xa, *tc_xattn, *tc_xact;
   float* tc_part;
   // host-buffer entry: side stream for the upload of the draft rows, and its two events

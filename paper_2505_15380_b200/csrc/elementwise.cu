@@ -58,8 +58,8 @@ __global__ void rope_table_kernel(const int32_t* __restrict__ len, RowMap rm,
                                   const double* __restrict__ inv_freq, int half,
                                   float* __restrict__ cs) {
   int m = blockIdx.x;
-  int bi = m / rm.R, r = m % rm.R;
-  double pos = (double)(len[rm.b0 + bi] + r);
+  const int2 br = row_at(rm, m);
+  double pos = (double)(len[br.x] + br.y);
   for (int j = threadIdx.x; j < half; j += blockDim.x) {
     double s, c;
     sincos(pos * inv_freq[j], &s, &c);
@@ -70,7 +70,7 @@ __global__ void rope_table_kernel(const int32_t* __restrict__ len, RowMap rm,
 
 void launch_rope_table(const int32_t* len, RowMap rm, const double* inv_freq, int half, float* cs,
                        cudaStream_t st) {
-  rope_table_kernel<<<rm.nb * rm.R, 64, 0, st>>>(len, rm, inv_freq, half, cs);
+  rope_table_kernel<<<row_count(rm), 64, 0, st>>>(len, rm, inv_freq, half, cs);
   count_launch();
 }
 
@@ -172,6 +172,49 @@ __global__ void advance_len_kernel(int32_t* len, int32_t* pending, int b, int ad
 void launch_advance_len(int32_t* len, int32_t* pending, int b, int add, const int32_t* ids,
                         int pending_index, cudaStream_t st) {
   advance_len_kernel<<<1, 1, 0, st>>>(len, pending, b, add, ids, pending_index);
+  count_launch();
+}
+
+// Rows of a prefill chunk: ids, (stream, r) of every row, the attention's tiles.
+__global__ void prefill_stage_kernel(const __grid_constant__ PrefillSegs P, const int32_t* __restrict__ ids,
+                                     int32_t* __restrict__ row_ids, int2* __restrict__ rows,
+                                     int4* __restrict__ tiles) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < P.n_rows) {
+    int q = 0;
+    while (q + 1 < P.n && i >= P.s[q + 1].m0) ++q;  // segments without rows share their m0: the last one wins,
+    while (P.s[q].count == 0) --q;                  // so step back to the one that has the row
+    const int r = i - P.s[q].m0;
+    row_ids[i] = ids[P.s[q].src + r];
+    rows[i] = make_int2(P.s[q].stream, r);
+  }
+  if (i < P.n_tiles) {
+    int q = 0;
+    while (q + 1 < P.n && i >= P.s[q + 1].tile0) ++q;
+    while (P.s[q].count == 0) --q;
+    const int r = (i - P.s[q].tile0) * P.tile_rows;
+    tiles[i] = make_int4(P.s[q].stream, P.s[q].m0 + r, r, min(P.tile_rows, P.s[q].count - r));
+  }
+}
+
+void launch_prefill_stage(const PrefillSegs& segs, const int32_t* ids, int32_t* row_ids, int2* rows, int4* tiles,
+                          cudaStream_t st) {
+  prefill_stage_kernel<<<(segs.n_rows + 127) / 128, 128, 0, st>>>(segs, ids, row_ids, rows, tiles);
+  count_launch();
+}
+
+// The chunk's rows are in the cache: lengths grow, prompts that end here leave their last id pending.
+__global__ void prefill_advance_kernel(const __grid_constant__ PrefillSegs P, const int32_t* __restrict__ ids,
+                                       int32_t* len, int32_t* pending) {
+  const int q = threadIdx.x;
+  if (q >= P.n) return;
+  len[P.s[q].stream] += P.s[q].count;
+  if (P.s[q].pend_src >= 0) pending[P.s[q].stream] = ids[P.s[q].pend_src];
+}
+
+void launch_prefill_advance(const PrefillSegs& segs, const int32_t* ids, int32_t* len, int32_t* pending,
+                            cudaStream_t st) {
+  prefill_advance_kernel<<<1, PREFILL_SEGS, 0, st>>>(segs, ids, len, pending);
   count_launch();
 }
 

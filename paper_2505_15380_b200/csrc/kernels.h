@@ -24,6 +24,10 @@ void launch_rmsnorm(int dtype, const float* h, const void* gain, float* out, int
 void launch_qkv_post(int dtype, const float* qkv, const float* cs, float* qrot, void* kv_layer,
                      const int32_t* len, RowMap rm, int cap, int Hq, int Hkv, int hd,
                      int32_t* status, cudaStream_t st);
+void launch_prefill_stage(const PrefillSegs& segs, const int32_t* ids, int32_t* row_ids, int2* rows, int4* tiles,
+                          cudaStream_t st);
+void launch_prefill_advance(const PrefillSegs& segs, const int32_t* ids, int32_t* len, int32_t* pending,
+                            cudaStream_t st);
 void launch_advance_len(int32_t* len, int32_t* pending, int b, int add, const int32_t* ids,
                         int pending_index, cudaStream_t st);
 

@@ -48,7 +48,7 @@ namespace ssd {
 
 constexpr int TC_TILE_ROWS = 128;                 // weight rows per tile = M of the MMA
 constexpr int TC_WBLOCK = TC_TILE_ROWS * 16 * 2;  // bytes of one (tile, k-step) weight block
-constexpr int TC_MAX_ROWS = 512;                  // token rows per forward (tensor-memory columns)
+constexpr int TC_MAX_ROWS = 2304;                 // token rows per forward (prefill chunks; chunks of <= 256 rows per CTA)
 constexpr int TC_THREADS = 256;                   // copy warp, MMA warp, six more; all eight run the epilogue
 
 enum TcEpilogue {
@@ -82,6 +82,26 @@ inline cudaError_t tc_launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, 
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
 }
+// The same with thread-block clusters of `cluster` CTAs along x.
+template <typename... KArgs, typename... Args>
+inline cudaError_t tc_launch_pdl_cluster(void (*kern)(KArgs...), dim3 grid, dim3 block, int cluster, size_t smem,
+                                         cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)cluster;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
+}
 #endif
 
 inline int tc_round16(int m) { return (m + 15) / 16 * 16; }
@@ -104,29 +124,31 @@ inline size_t tc_act_bytes(int M, int K) {
   const TcChunks c = tc_chunks(M);
   return (size_t)((K + 15) / 16) * c.n * c.rows * 64;
 }
-// Byte offset of element (part, t, k) of a packed operand with chunks of Mc rows and KS k-steps.
+// Where element (part, t, k) of a packed operand is: in chunk t / Mc, at
+//   (t % Mc) * 16 + (k / 16) * kstep + ((k / 8) % 2) * half + part * part_off + (k % 8) * 2.
+// Two arrangements: k-steps holding both parts (one instruction multiplies both), or a chunk's
+// leading parts followed by its remainders (each CTA of a pair takes one part: tc_prefill.cu).
+struct ActLay {
+  int Mc;
+  uint32_t kstep, half, part_off;
+  uint32_t chunk;  // bytes per chunk
 #ifdef __CUDACC__
-__host__ __device__
+  __device__ __forceinline__ uint8_t* row(uint8_t* base, int t) const {
+    const int ch = t / Mc;
+    return base + (size_t)ch * chunk + (size_t)(t - ch * Mc) * 16;
+  }
+  __device__ __forceinline__ size_t col(int k) const {
+    return (size_t)(k >> 4) * kstep + ((k >> 3) & 1) * half + (k & 7) * 2;
+  }
 #endif
-inline size_t tc_act_off(int Mc, int KS, int part, int t, int k) {
-  const int ch = t / Mc, tl = t - ch * Mc;
-  return ((size_t)ch * KS + (size_t)(k >> 4)) * ((size_t)Mc * 64) + (size_t)((k >> 3) & 1) * ((size_t)Mc * 32) +
-         (size_t)part * ((size_t)Mc * 16) + (size_t)tl * 16 + (size_t)(k & 7) * 2;
+};
+inline ActLay tc_act_lay(int Mc, int K) {
+  const uint32_t KS = (uint32_t)(K + 15) / 16, m = (uint32_t)Mc;
+  return ActLay{Mc, m * 64, m * 32, m * 16, KS * m * 64};
 }
-// The same offset in two terms, for code that writes many columns of one row: the row's term
-// (its chunk and its place in it) and the column's.
-#ifdef __CUDACC__
-__host__ __device__
-#endif
-inline size_t tc_act_row_off(int Mc, int KS, int t) {
-  const int ch = t / Mc, tl = t - ch * Mc;
-  return (size_t)ch * KS * ((size_t)Mc * 64) + (size_t)tl * 16;
-}
-#ifdef __CUDACC__
-__host__ __device__
-#endif
-inline size_t tc_act_col_off(int Mc, int k) {
-  return (size_t)(k >> 4) * ((size_t)Mc * 64) + (size_t)((k >> 3) & 1) * ((size_t)Mc * 32) + (size_t)(k & 7) * 2;
+inline ActLay tc_act_lay_parts(int Mc, int K) {
+  const uint32_t KS = (uint32_t)(K + 15) / 16, m = (uint32_t)Mc;
+  return ActLay{Mc, m * 32, m * 16, KS * m * 32, KS * m * 64};
 }
 // Weight-row tiles per CTA: two where the token rows come in chunks (more than 256 rows) and the
 // projection is long (many tiles, or a deep K): the tiles then share the activation blocks the
@@ -147,12 +169,26 @@ inline int tc_ksplit(int n_rows, int K, int M, int n_sm) {
   return s < 1 ? 1 : s;
 }
 
+// Row chunks of a prefill: at most 64 rows each.  Every row is summed exactly as in a forward of up
+// to 128 rows - the same K slices, even and odd k-steps and the two bf16 parts in accumulators of
+// their own - so that a prompt's keys and values do not depend on how many other rows its chunk
+// happened to hold.
+constexpr int TC_PREFILL_CHUNK = 64;
+inline TcChunks tc_prefill_chunks(int M) {
+  const int Mpad = tc_round16(M);
+  TcChunks c;
+  c.n = (Mpad + TC_PREFILL_CHUNK - 1) / TC_PREFILL_CHUNK;
+  c.rows = tc_round16((Mpad + c.n - 1) / c.n);
+  return c;
+}
+
 struct TcGemm {
   const uint8_t* w;   // packed weights of the projection
   const uint8_t* a;   // packed activations
   int n_rows, K;      // weight rows, input columns
   int M;              // token rows
   int ksplit;
+  int mc = 0;         // launch_tc_prefill_gemm: rows per chunk of the operands
   int epi;
   float* part;        // TC_EPI_PARTIAL: [ksplit][Mpad][tiles * 128]
   float* out;         // TC_EPI_STORE
@@ -160,6 +196,28 @@ struct TcGemm {
   uint8_t* act_out;   // TC_EPI_SWIGLU: packed operand of n_rows / 2 columns
   int32_t* status;
 };
+
+// Whether a projection of at most 128 token rows that runs as `ctas` CTAs has an SM's whole tensor
+// memory: even and odd k-steps then accumulate into two column sets.  (Two CTAs share an SM where
+// their number exceeds the SMs by a little.)
+inline bool tc_dual_sets(int ctas, int n_sm) { return !(ctas > n_sm && ctas <= 2 * n_sm); }
+
+// tc_prefill.cu: a projection of a prefill chunk, g.ksplit slices added within a CTA.
+enum PfEpilogue {
+  PF_EPI_BIAS = 0,      // out[t, n] = bias[n] + acc
+  PF_EPI_RESIDUAL = 1,  // out[t, n] += acc
+  PF_EPI_SWIGLU = 2,    // act_out: packed SiLU(gate) * up (arranged as act_out_lay says)
+  PF_EPI_PARTIAL = 3    // out[slice][Mpad][tiles * 128] = the slice's sums
+};
+// Over how many work items the slices are shared out: as many as it takes to occupy the pairs of SMs.
+// One: the slices are added within the CTA.
+inline int tc_prefill_groups(int n_rows, int M, int nslice, int n_sm) {
+  const int items = (n_rows + 2 * TC_TILE_ROWS - 1) / (2 * TC_TILE_ROWS) * ((tc_prefill_chunks(M).n + 1) / 2);
+  const int g = n_sm / 2 / items;
+  return g < 2 ? 1 : (g < nslice ? g : nslice);
+}
+cudaError_t launch_tc_prefill_gemm(const TcGemm& g, int epi, const bf16* bias, float* out, int n_sm, cudaStream_t st,
+                                   ActLay act_out_lay = ActLay());
 
 // tc_gemm.cu
 cudaError_t tc_pack_weights(const bf16* w_rowmajor, int n_rows, int K, uint8_t* packed, cudaStream_t st);
@@ -170,7 +228,7 @@ cudaError_t launch_tc_gemm(const TcGemm& g, cudaStream_t st);
 // h[m, :] += sum of `nsplit` partial projections (part may be null); then the RMS norm of the row
 // times `gain`, written as a packed operand (hi + lo) of d columns.  h_in may differ from h (the
 // first layer reads the embedding rows).
-void launch_tc_norm_pack(float* h, const float* part, int nsplit, int ld_part, int M, int d,
+void launch_tc_norm_pack(float* h, const float* part, int nsplit, int ld_part, int M, ActLay lay, int d,
                          const bf16* gain, float eps, uint8_t* apack, cudaStream_t st);
 // Packs fp32 rows x[M, K] as an operand (used by tests of the projection kernel).
 void launch_tc_pack_rows(const float* x, int M, int K, uint8_t* apack, cudaStream_t st);
@@ -189,6 +247,8 @@ void launch_tc_qkv_post(const float* part, int nsplit, int ld_part, int Mpad, co
 void launch_page_ensure(const int32_t* len, RowMap rm, int32_t* page_table, int32_t* pages_used,
                         int32_t* free_stack, int32_t* free_top, int max_pages, int32_t* status,
                         cudaStream_t st);
+void launch_page_ensure_segs(const int32_t* len, const PrefillSegs& segs, int32_t* page_table, int32_t* pages_used,
+                             int32_t* free_stack, int32_t* free_top, int max_pages, int32_t* status, cudaStream_t st);
 void launch_page_release(const int32_t* len, int B, int32_t* page_table, int32_t* pages_used,
                          int32_t* free_stack, int32_t* free_top, int max_pages, cudaStream_t st);
 
@@ -196,7 +256,7 @@ void launch_page_release(const int32_t* len, int B, int32_t* page_table, int32_t
 // split over the keys; the merged result is written as the packed operand of the O projection.
 cudaError_t launch_tc_attention(const float* qrot, const bf16* kv_layer, const int32_t* len, RowMap rm,
                                 int cap, int Hq, int Hkv, int hd, float* part, int nsplit,
-                                int keys_per_split, uint8_t* apack_out, int Mpad,
+                                int keys_per_split, uint8_t* apack_out, ActLay lay,
                                 const int32_t* page_table, int max_pages, int which_kernel, int32_t* status,
                                 cudaStream_t st);
 int tc_attention_ctas_per_sm(int hd);  // CTAs of the attention kernel an SM holds at once

@@ -63,7 +63,8 @@ template <int HD>
 __global__ void __launch_bounds__(TA_WARPS * 32)
 tc_attn_kernel(const float* __restrict__ qrot, const bf16* __restrict__ kv_layer, const int32_t* __restrict__ len,
                RowMap rm, int cap, int Hq, int Hkv, int n_rowgroups, float* __restrict__ part, int nsplit,
-               int keys_per_split, const int32_t* __restrict__ page_table, int max_pages) {
+               int keys_per_split, const int32_t* __restrict__ page_table, int max_pages,
+               uint8_t* __restrict__ apack, ActLay lay) {
   constexpr int ROWB = HD * 2 + 16;   // padded K / V row: conflict-free matrix loads
   constexpr int KSTEPS = HD / 16;
   constexpr int DT = HD / 8;
@@ -74,10 +75,20 @@ tc_attn_kernel(const float* __restrict__ qrot, const bf16* __restrict__ kv_layer
   uint4* q_s = reinterpret_cast<uint4*>(smem + 4 * TILE_BYTES);  // [warp][kstep][lane][hi 4 words | lo 4 words]
 
   const int sp = blockIdx.x, gk = blockIdx.y / n_rowgroups, rg = blockIdx.y % n_rowgroups, bi = blockIdx.z;
-  const int b = rm.b0 + bi, R = rm.R, G = Hq / Hkv, NQ = G * R;
+  const int G = Hq / Hkv;
   tc_pdl_trigger();
   tc_pdl_wait();
-  const int L = len[b], total = min(L + R, cap);
+  // the rows of this work item: R rows of stream b, from row mbase of the forward and row rel of the
+  // stream's new rows on
+  int b = rm.b0 + bi, R = rm.R, mbase = bi * rm.R, rel = 0;
+  if (rm.tiles) {
+    const int4 tl = rm.tiles[bi];
+    b = tl.x;
+    mbase = tl.y;
+    rel = tl.z;
+    R = tl.w;
+  }
+  const int NQ = G * R, L = len[b] + rel, total = min(L + R, cap);
   const int k_begin = sp * keys_per_split;
   if (k_begin >= total) return;
   const int k_end = min(k_begin + keys_per_split, total);
@@ -113,7 +124,7 @@ tc_attn_kernel(const float* __restrict__ qrot, const bf16* __restrict__ kv_layer
   const bool ok0 = i0 < NQ, ok1 = i1 < NQ;
   const int r0 = ok0 ? i0 % R : 0, r1 = ok1 ? i1 % R : 0;
   const int h0 = gk * G + (ok0 ? i0 / R : 0), h1 = gk * G + (ok1 ? i1 / R : 0);
-  const int m0 = bi * R + r0, m1 = bi * R + r1;
+  const int m0 = mbase + r0, m1 = mbase + r1;
   {  // q as A fragments (bf16 leading part + remainder), each lane its own
     const float* q0 = qrot + ((size_t)m0 * Hq + h0) * HD;
     const float* q1 = qrot + ((size_t)m1 * Hq + h1) * HD;
@@ -267,6 +278,25 @@ tc_attn_kernel(const float* __restrict__ qrot, const bf16* __restrict__ kv_layer
     l_run[hh] += __shfl_xor_sync(0xffffffffu, l_run[hh], 1);
     l_run[hh] += __shfl_xor_sync(0xffffffffu, l_run[hh], 2);
   }
+  if (apack) {  // one key range per row: this is the result, written as the operand of the O projection
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+      if (hh ? ok1 : ok0) {
+        const float inv = 1.f / l_run[hh];
+        uint8_t* row = lay.row(apack, hh ? m1 : m0);
+        const int k0 = (hh ? h1 : h0) * HD + 2 * t;
+#pragma unroll
+        for (int dt = 0; dt < DT; ++dt) {
+          uint32_t hi, lo;
+          split2(o[dt][2 * hh] * inv, o[dt][2 * hh + 1] * inv, hi, lo);
+          uint8_t* e = row + lay.col(k0 + dt * 8);
+          *reinterpret_cast<uint32_t*>(e) = hi;
+          *reinterpret_cast<uint32_t*>(e + lay.part_off) = lo;
+        }
+      }
+    }
+    return;
+  }
   if (ok0) {
     float* dst = part + (((size_t)m0 * Hq + h0) * nsplit + sp) * (HD + 2);
 #pragma unroll
@@ -287,64 +317,84 @@ tc_attn_kernel(const float* __restrict__ qrot, const bf16* __restrict__ kv_layer
   }
 }
 
-// Grid (query head, row).  Merges the key splits of one (row, head) and writes the normalised
-// output as columns h * HD .. of the packed operand.
+// One warp per (row, query head), MERGE_WARPS to a CTA.  Merges the key splits and writes the
+// normalised output as columns h * HD .. of the packed operand.  Lane s holds the statistics of
+// split s (and of s + 32, ..); the splits' outputs are added in order, eight loads in flight.
+constexpr int MERGE_WARPS = 4;
 template <int HD>
-__global__ void tc_attn_merge_kernel(const float* __restrict__ part, const int32_t* __restrict__ len, RowMap rm,
-                                     int cap, int Hq, int nsplit, int keys_per_split,
-                                     uint8_t* __restrict__ apack, int Mc) {
-  const int h = blockIdx.x, m = blockIdx.y;
-  const int bi = m / rm.R, b = rm.b0 + bi;
+__global__ void __launch_bounds__(MERGE_WARPS * 32)
+tc_attn_merge_kernel(const float* __restrict__ part, const int32_t* __restrict__ len, RowMap rm, int n_pairs,
+                     int cap, int Hq, int nsplit, int keys_per_split, uint8_t* __restrict__ apack, ActLay lay) {
+  constexpr int NP = HD >= 64 ? HD / 64 : 1;  // column pairs per lane
+  const int lane = threadIdx.x & 31, pair = blockIdx.x * MERGE_WARPS + (threadIdx.x >> 5);
   tc_pdl_trigger();
   tc_pdl_wait();
-  const int total = min(len[b] + rm.R, cap);
-  const int ns = (total + keys_per_split - 1) / keys_per_split;
-  const float* src = part + ((size_t)m * Hq + h) * nsplit * (HD + 2);
-  __shared__ float s_m[128], s_w[128];  // running max and sum of each split, then its weight
-  for (int s = threadIdx.x; s < ns; s += blockDim.x) {
-    s_m[s] = __ldcg(src + s * (HD + 2) + HD);
-    s_w[s] = __ldcg(src + s * (HD + 2) + HD + 1);
+  if (pair >= n_pairs) return;  // uniform per warp
+  const int m = pair / Hq, h = pair - m * Hq;
+  int b = rm.b0 + m / rm.R, last = rm.R;
+  if (rm.rows) {  // the splits that the row's work item wrote: up to its last row
+    const int2 br = rm.rows[m];
+    b = br.x;
+    last = br.y + 1;
   }
-  __syncthreads();
+  const int total = min(len[b] + last, cap), ns = (total + keys_per_split - 1) / keys_per_split;
+  const float* src = part + (size_t)pair * nsplit * (HD + 2);
   float m_tot = -CUDART_INF_F;
-  for (int s = 0; s < ns; ++s) m_tot = fmaxf(m_tot, s_m[s]);
+  for (int s0 = 0; s0 < ns; s0 += 32)
+    if (s0 + lane < ns) m_tot = fmaxf(m_tot, __ldcg(src + (size_t)(s0 + lane) * (HD + 2) + HD));
+  m_tot = warp_max(m_tot);
   float denom = 0.f;
-  for (int s = 0; s < ns; ++s) {  // fixed order
-    const float e = s_m[s] == -CUDART_INF_F ? 0.f : __expf(s_m[s] - m_tot);
-    denom = fmaf(e, s_w[s], denom);
-  }
-  __syncthreads();
-  for (int s = threadIdx.x; s < ns; s += blockDim.x) s_w[s] = s_m[s] == -CUDART_INF_F ? 0.f : __expf(s_m[s] - m_tot);
-  __syncthreads();
-  const float inv = 1.f / denom;
-  uint8_t* arow = apack + tc_act_row_off(Mc, (Hq * HD + 15) >> 4, m);
-  for (int d = threadIdx.x * 2; d < HD; d += blockDim.x * 2) {
-    float o0 = 0.f, o1 = 0.f;
-#pragma unroll 4
-    for (int s = 0; s < ns; ++s) {  // fixed order
-      const float2 v = __ldcg(reinterpret_cast<const float2*>(src + s * (HD + 2) + d));
-      o0 = fmaf(s_w[s], v.x, o0);
-      o1 = fmaf(s_w[s], v.y, o1);
+  float2 o[NP];
+#pragma unroll
+  for (int p = 0; p < NP; ++p) o[p] = make_float2(0.f, 0.f);
+  for (int s0 = 0; s0 < ns; s0 += 32) {
+    float e = 0.f, l = 0.f;  // weight and sum of split s0 + lane
+    if (s0 + lane < ns) {
+      const float2 ml = __ldcg(reinterpret_cast<const float2*>(src + (size_t)(s0 + lane) * (HD + 2) + HD));
+      e = ml.x == -CUDART_INF_F ? 0.f : __expf(ml.x - m_tot);
+      l = ml.y;
     }
-    o0 *= inv;
-    o1 *= inv;
-    const int k = h * HD + d;
-    const __nv_bfloat162 hi = __floats2bfloat162_rn(o0, o1);
-    const __nv_bfloat162 lo = __floats2bfloat162_rn(o0 - __low2float(hi), o1 - __high2float(hi));
-    uint8_t* e = arow + tc_act_col_off(Mc, k);
-    *reinterpret_cast<__nv_bfloat162*>(e) = hi;
-    *reinterpret_cast<__nv_bfloat162*>(e + (size_t)Mc * 16) = lo;
+    const int n = min(32, ns - s0);
+#pragma unroll 8
+    for (int s = 0; s < n; ++s) {  // fixed order
+      const float es = __shfl_sync(0xffffffffu, e, s), ls = __shfl_sync(0xffffffffu, l, s);
+      denom = fmaf(es, ls, denom);
+      const float* row = src + (size_t)(s0 + s) * (HD + 2);
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        const int d = p * 64 + lane * 2;
+        if (d < HD) {
+          const float2 v = __ldcg(reinterpret_cast<const float2*>(row + d));
+          o[p].x = fmaf(es, v.x, o[p].x);
+          o[p].y = fmaf(es, v.y, o[p].y);
+        }
+      }
+    }
+  }
+  const float inv = 1.f / denom;
+  uint8_t* arow = lay.row(apack, m);
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    const int d = p * 64 + lane * 2;
+    if (d < HD) {
+      uint32_t hi, lo;
+      split2(o[p].x * inv, o[p].y * inv, hi, lo);
+      uint8_t* e = arow + lay.col(h * HD + d);
+      *reinterpret_cast<uint32_t*>(e) = hi;
+      *reinterpret_cast<uint32_t*>(e + lay.part_off) = lo;
+    }
   }
 }
 
 template <int HD>
 cudaError_t launch_t(const float* qrot, const bf16* kv_layer, const int32_t* len, RowMap rm, int cap, int Hq,
-                     int Hkv, float* part, int nsplit, int keys_per_split, uint8_t* apack_out, int Mpad,
+                     int Hkv, float* part, int nsplit, int keys_per_split, uint8_t* apack_out, ActLay lay,
                      const int32_t* page_table, int max_pages, int which_kernel, int32_t* status, cudaStream_t st) {
-  const int NQ = (Hq / Hkv) * rm.R, n_rowgroups = (NQ + TA_WARPS * 16 - 1) / (TA_WARPS * 16);
+  const int NQ = rm.tiles ? 1 : (Hq / Hkv) * rm.R;  // a listed tile is one row group
+  const int n_rowgroups = (NQ + TA_WARPS * 16 - 1) / (TA_WARPS * 16), items = rm.tiles ? rm.n_tiles : rm.nb;
   const size_t smem = (size_t)4 * TA_TILE * (HD * 2 + 16) + (size_t)TA_WARPS * (HD / 16) * 32 * 32;
   cudaError_t e;
-  const bool t5 = HD >= 64 && (which_kernel == 2 || (which_kernel == 0 && keys_per_split >= TC_ATTN5_MIN_KEYS));
+  const bool t5 = HD >= 64 && !rm.tiles && (which_kernel == 2 || (which_kernel == 0 && keys_per_split >= TC_ATTN5_MIN_KEYS));
   if (t5) {  // tcgen05 contractions
     e = launch_tc_attention5(qrot, kv_layer, len, rm, cap, Hq, Hkv, HD, part, nsplit, keys_per_split, page_table,
                              max_pages, status, st);
@@ -353,14 +403,17 @@ cudaError_t launch_t(const float* qrot, const bf16* kv_layer, const int32_t* len
     auto kern = tc_attn_kernel<HD>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = tc_launch_pdl(kern, dim3(nsplit, Hkv * n_rowgroups, rm.nb), dim3(TA_WARPS * 32), smem, st, qrot, kv_layer, len,
-                      rm, cap, Hq, Hkv, n_rowgroups, part, nsplit, keys_per_split, page_table, max_pages);
+    e = tc_launch_pdl(kern, dim3(nsplit, Hkv * n_rowgroups, items), dim3(TA_WARPS * 32), smem, st, qrot, kv_layer, len,
+                      rm, cap, Hq, Hkv, n_rowgroups, part, nsplit, keys_per_split, page_table, max_pages,
+                      nsplit == 1 ? apack_out : nullptr, lay);
     if (e != cudaSuccess) return e;
     count_launch();
+    if (nsplit == 1) return cudaGetLastError();
   }
-  e = tc_launch_pdl(tc_attn_merge_kernel<HD>, dim3(Hq, rm.nb * rm.R), dim3(HD / 2 < 32 ? 32 : HD / 2), 0, st,
-                    (const float*)part, len, rm, cap, Hq, nsplit, keys_per_split, apack_out,
-                    tc_chunks(rm.nb * rm.R).rows);
+  const int n_pairs = row_count(rm) * Hq;
+  e = tc_launch_pdl(tc_attn_merge_kernel<HD>, dim3((n_pairs + MERGE_WARPS - 1) / MERGE_WARPS), dim3(MERGE_WARPS * 32), 0,
+                    st, (const float*)part, len, rm, n_pairs, cap, Hq, nsplit, keys_per_split, apack_out,
+                    lay);
   if (e != cudaSuccess) return e;
   count_launch();
   return cudaGetLastError();
@@ -372,14 +425,14 @@ int tc_attention_ctas_per_sm(int) { return 2; }
 
 cudaError_t launch_tc_attention(const float* qrot, const bf16* kv_layer, const int32_t* len, RowMap rm,
                                 int cap, int Hq, int Hkv, int hd, float* part, int nsplit,
-                                int keys_per_split, uint8_t* apack_out, int Mpad,
+                                int keys_per_split, uint8_t* apack_out, ActLay lay,
                                 const int32_t* page_table, int max_pages, int which_kernel, int32_t* status,
                                 cudaStream_t st) {
   if (page_table && keys_per_split % TC_PAGE_TOKENS) return cudaErrorInvalidValue;
   switch (hd) {
-    case 32: return launch_t<32>(qrot, kv_layer, len, rm, cap, Hq, Hkv, part, nsplit, keys_per_split, apack_out, Mpad, page_table, max_pages, which_kernel, status, st);
-    case 64: return launch_t<64>(qrot, kv_layer, len, rm, cap, Hq, Hkv, part, nsplit, keys_per_split, apack_out, Mpad, page_table, max_pages, which_kernel, status, st);
-    case 128: return launch_t<128>(qrot, kv_layer, len, rm, cap, Hq, Hkv, part, nsplit, keys_per_split, apack_out, Mpad, page_table, max_pages, which_kernel, status, st);
+    case 32: return launch_t<32>(qrot, kv_layer, len, rm, cap, Hq, Hkv, part, nsplit, keys_per_split, apack_out, lay, page_table, max_pages, which_kernel, status, st);
+    case 64: return launch_t<64>(qrot, kv_layer, len, rm, cap, Hq, Hkv, part, nsplit, keys_per_split, apack_out, lay, page_table, max_pages, which_kernel, status, st);
+    case 128: return launch_t<128>(qrot, kv_layer, len, rm, cap, Hq, Hkv, part, nsplit, keys_per_split, apack_out, lay, page_table, max_pages, which_kernel, status, st);
   }
   return cudaErrorInvalidValue;
 }

@@ -466,7 +466,7 @@ cudaError_t launch_tc_gemm(const TcGemm& g, cudaStream_t st) {
       n_sm = 148;
   }
   const int ctas = grid_x * g.ksplit * ch.n;
-  const bool two_per_sm = p.Mpad <= 128 && ctas > n_sm && ctas <= 2 * n_sm;  // 2 x 256 columns
+  const bool two_per_sm = ch.n == 1 && p.Mpad <= 128 && !tc_dual_sets(ctas, n_sm);  // 2 x 256 columns
   const size_t budget = two_per_sm ? 100 * 1024 : 216 * 1024;
   p.sk = 4;
   while (p.sk > 1 && 3 * p.sk * per_ks > budget) p.sk >>= 1;
@@ -477,7 +477,7 @@ cudaError_t launch_tc_gemm(const TcGemm& g, cudaStream_t st) {
   const int op_rows = p.wide ? 2 * p.Mc : p.ntile * p.Mc;  // accumulator columns
   p.nchunks = p.wide ? (op_rows + 255) / 256 : 1;
   p.chunk_n = p.wide ? tc_round16((op_rows + p.nchunks - 1) / p.nchunks) : p.Mc;
-  p.dual = p.wide && 4 * p.Mc <= 512 && !two_per_sm;  // two CTAs on an SM have 256 columns each
+  p.dual = p.wide && 4 * p.Mc <= 512 && tc_dual_sets(grid_x * g.ksplit, n_sm);  // two CTAs on an SM have 256 columns each
   p.tmem_cols = 32;
   while (p.tmem_cols < (p.dual ? 2 : 1) * op_rows) p.tmem_cols <<= 1;
   const size_t smem = (size_t)p.stages * p.sk * per_ks + sizeof(TcShared) + 64;
