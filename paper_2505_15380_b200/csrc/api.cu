@@ -244,7 +244,9 @@ WsPlan plan_ws(const ssd_model_config& c, int B, int max_gamma, int cap, int n_p
         const size_t row_bytes = (size_t)mp * tiles * TC_TILE_ROWS * 4;
         const int nsl = tc_ksplit(rows[i], ks[i], TC_PREFILL_CHUNK, n_sm);
         part = std::max(part, tc_prefill_groups(rows[i], mp, nsl, n_sm) > 1 ? nsl * row_bytes : row_bytes);
-        if (mp <= Mdec) part = std::max(part, tc_ksplit(rows[i], ks[i], mp, n_sm) * row_bytes);
+        if (mp > TC_PAIR_MIN_ROWS && mp <= Mdec)
+          part = std::max(part, tc_prefill_groups(rows[i], mp, (ks[i] + 63) / 64, n_sm) * row_bytes);
+        else if (mp <= Mdec) part = std::max(part, tc_ksplit(rows[i], ks[i], mp, n_sm) * row_bytes);
       }
     }
     p.tc_part = take(part);
@@ -353,14 +355,16 @@ int forward_tc(const ssd_model* m, ssd_streams* s, RowMap rm, float* logits_out,
   const int qd = c.n_q_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim, F = c.d_ffn, nq = qd + 2 * kvd;
   const int n_sm = m->tc.n_sm;
   auto ld_of = [](int rows) { return (rows + TC_TILE_ROWS - 1) / TC_TILE_ROWS * TC_TILE_ROWS; };
-  const int Mks = rm.rows ? TC_PREFILL_CHUNK : M;
-  const int ks_qkv = tc_ksplit(nq, d, Mks, n_sm), ks_o = tc_ksplit(d, qd, Mks, n_sm), ks_d = tc_ksplit(d, F, Mks, n_sm);
+  // a prefill's rows are summed as a forward of max_rows rows would sum them, whatever the chunk holds
+  const bool seg = rm.rows != nullptr, pairs = seg || M > TC_PAIR_MIN_ROWS;
+  auto slices = [&](int rows, int K) {
+    return seg ? tc_ksplit(rows, K, TC_PREFILL_CHUNK, n_sm) : pairs ? tc_prefill_groups(rows, M, (K + 63) / 64, n_sm) : tc_ksplit(rows, K, M, n_sm);
+  };
+  const int ks_qkv = slices(nq, d), ks_o = slices(d, qd), ks_d = slices(d, F);
   // key splits of the attention: whole 64-key tiles, and no more CTAs in all than the SMs hold
   // at once (a second, partly filled wave would cost as much as the first)
   const int G = c.n_q_heads / c.n_kv_heads, rowgroups = (G * rm.R + 63) / 64;
-  // a prefill's rows are summed as a forward of max_rows rows would sum them, whatever the chunk holds
-  const bool seg = rm.rows != nullptr;
-  const int Mc = seg ? tc_prefill_chunks(M).rows : tc_chunks(M).rows;
+  const int Mc = pairs ? tc_prefill_chunks(M).rows : tc_chunks(M).rows;
   long long want = ((long long)tc_attention_ctas_per_sm(c.head_dim) * n_sm) /
                    (seg ? (long long)c.n_kv_heads * ((G * s->max_rows + 63) / 64)
                         : (long long)rm.nb * c.n_kv_heads * rowgroups);  // splits that still fit one wave
@@ -378,12 +382,12 @@ int forward_tc(const ssd_model* m, ssd_streams* s, RowMap rm, float* logits_out,
                        s->status, st);
   launch_embed(1, m->embed, c.vocab_out + c.vocab_text, d, s->row_ids, M, s->h, s->status, st);
   launch_rope_table(s->len, rm, m->inv_freq, c.head_dim / 2, s->rope_cs, st);
-  // prefill: whether a projection's slices are added within its CTAs, or written out one by one
-  const bool in_qkv = seg && tc_prefill_groups(nq, M, ks_qkv, n_sm) == 1, in_o = seg && tc_prefill_groups(d, M, ks_o, n_sm) == 1,
-             in_d = seg && tc_prefill_groups(d, M, ks_d, n_sm) == 1;
-  auto lay = [&](int K) { return seg ? tc_act_lay_parts(Mc, K) : tc_act_lay(Mc, K); };
+  // pair kernel: whether a projection's slices are added within its CTAs, or written out one by one
+  const bool in_qkv = pairs && tc_prefill_groups(nq, M, ks_qkv, n_sm) == 1, in_o = pairs && tc_prefill_groups(d, M, ks_o, n_sm) == 1,
+             in_d = pairs && tc_prefill_groups(d, M, ks_d, n_sm) == 1;
+  auto lay = [&](int K) { return pairs ? tc_act_lay_parts(Mc, K) : tc_act_lay(Mc, K); };
   auto gemm = [&](const TcGemm& q, bool in_cta, int epi, const void* bias, float* out) {
-    if (!seg) return launch_tc_gemm(q, st);
+    if (!pairs) return launch_tc_gemm(q, st);
     return launch_tc_prefill_gemm(q, in_cta || epi == PF_EPI_SWIGLU ? epi : PF_EPI_PARTIAL, (const bf16*)bias,
                                   in_cta ? out : q.part, n_sm, st, lay(q.n_rows / 2));
   };
@@ -391,7 +395,7 @@ int forward_tc(const ssd_model* m, ssd_streams* s, RowMap rm, float* logits_out,
   int nsp = 0, ldp = 0;
   TcGemm g{};
   g.M = M;
-  g.mc = seg ? Mc : 0;
+  g.mc = Mc;
   g.status = s->status;
   for (int l = 0; l < c.n_layers; ++l) {
     const LayerW& w = m->layers[l];
@@ -423,7 +427,7 @@ int forward_tc(const ssd_model* m, ssd_streams* s, RowMap rm, float* logits_out,
     launch_tc_norm_pack(s->h, part, nsp, ldp, M, lay(d), d, (const bf16*)m->norm_f, c.rms_eps, s->tc_xa, st);
     g.w = m->tc.head; g.a = s->tc_xa; g.n_rows = c.vocab_out; g.K = d; g.ksplit = 1; g.epi = TC_EPI_STORE;
     g.out = logits_out; g.ldo = c.vocab_out;
-    SSD_CUDA(launch_tc_gemm(g, st));
+    SSD_CUDA(gemm(g, pairs, PF_EPI_BIAS, nullptr, logits_out));
   }
   SSD_CUDA(cudaGetLastError());
   return SSD_OK;

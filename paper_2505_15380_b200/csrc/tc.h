@@ -182,6 +182,10 @@ inline TcChunks tc_prefill_chunks(int M) {
   return c;
 }
 
+// Verify forwards of more rows than this take the pair kernel too (tc_prefill.cu), with no more K
+// slices than it takes to occupy the chip.
+constexpr int TC_PAIR_MIN_ROWS = 128;
+
 struct TcGemm {
   const uint8_t* w;   // packed weights of the projection
   const uint8_t* a;   // packed activations

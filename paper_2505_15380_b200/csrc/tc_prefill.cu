@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) tc_prefill_gemm_kernel(const __
       float acc[2][32];
       {
         float b = 0.f;
-        if (EPI == PF_EPI_BIAS && n < P.n_rows) b = __bfloat162float(P.bias[n]);
+        if (EPI == PF_EPI_BIAS && P.bias && n < P.n_rows) b = __bfloat162float(P.bias[n]);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
 #pragma unroll
