@@ -64,8 +64,8 @@ struct ArenaPlan {
       f_gains;
   // weights packed for the tensor-core projections of batched forwards (bf16 models only)
   bool tc;
-  std::vector<LayerOff> tc_layers;  // w_qkv, w_o, w_gu, w_d used
-  size_t tc_head;
+  std::vector<LayerOff> tc_layers, ch_layers;  // w_qkv, w_o, w_gu, w_d used
+  size_t tc_head, ch_head;
 };
 
 // CTAs of the persistent kernel: one per SM of the current device (148 when none is present, the
@@ -128,6 +128,14 @@ ArenaPlan plan_arena(const ssd_model_config& c, const FastPlan* fp = nullptr) {
       L.w_d = take(tc_weight_bytes((int)d, (int)F));
     }
     p.tc_head = take(tc_weight_bytes(c.vocab_out, (int)d));
+    p.ch_layers.resize(c.n_layers);
+    for (auto& L : p.ch_layers) {
+      L.w_qkv = take(chain_weight_bytes((int)(qd + 2 * kvd), (int)d));
+      L.w_o = take(chain_weight_bytes((int)d, (int)qd));
+      L.w_gu = take(chain_weight_bytes((int)(2 * F), (int)d));
+      L.w_d = take(chain_weight_bytes((int)d, (int)F));
+    }
+    p.ch_head = take(chain_weight_bytes(c.vocab_out, (int)d));
   }
   p.total = off;
   return p;
@@ -145,7 +153,7 @@ struct WsPlan {
   size_t h, qkv, qrot, rope_cs, part, logits, row_stats, xn, attn_out, act;
   size_t st_tokens, st_k, st_y, st_probs, st_uni;
   size_t hfix, flags, epoch_base, xa, xb, xd, xq, ssq_a, ssq_b;
-  size_t tc_rowmap, tc_tiles, tc_xa, tc_xattn, tc_xact, tc_part;
+  size_t ch_ssq_a, ch_ssq_b, tc_rowmap, tc_tiles, tc_xa, tc_xattn, tc_xact, tc_part;
   size_t attn_part, attn_cnt;
   size_t page_table, pages_used, free_stack, free_top;
   size_t total;
@@ -220,8 +228,11 @@ WsPlan plan_ws(const ssd_model_config& c, int B, int max_gamma, int cap, int n_p
     p.free_stack = take((size_t)n_pages * 4);
     p.free_top = take(4);
   }
+  p.ch_ssq_a = p.ch_ssq_b = 0;
   p.tc_xa = p.tc_xattn = p.tc_xact = p.tc_part = p.tc_rowmap = p.tc_tiles = 0;
   if (MT > FAST_MAX_T) {
+    p.ch_ssq_a = take((size_t)FAST_MAX_CTAS * TC_CHAIN_ROWS * 4);
+    p.ch_ssq_b = take((size_t)FAST_MAX_CTAS * TC_CHAIN_ROWS * 4);
     p.tc_rowmap = take(MT * sizeof(int2));
     p.tc_tiles = take((MT + PREFILL_SEGS) * sizeof(int4));
     const int Mpad = tc_round16((int)MT), Mdec = tc_round16((int)M), n_sm = fast_cta_count();
@@ -348,6 +359,102 @@ bool use_tc(const ssd_model* m, const ssd_streams* s, RowMap rm) {
   return m->tc.enabled && s->path == 0 && s->tc_part && M > FAST_MAX_T && M <= s->tc_rows;
 }
 
+// Key splits of the batched attention: whole 64-key tiles, and no more CTAs in all than the SMs hold
+// at once (a second, partly filled wave would cost as much as the first).
+struct KeySplit {
+  int n, keys;
+};
+KeySplit key_split(const ssd_model* m, const ssd_streams* s, RowMap rm) {
+  const ssd_model_config& c = m->cfg;
+  const int G = c.n_q_heads / c.n_kv_heads, rowgroups = (G * rm.R + 63) / 64;
+  // a prefill's keys are split as those of a forward of max_rows rows, whatever the chunk holds
+  long long want = ((long long)tc_attention_ctas_per_sm(c.head_dim) * m->tc.n_sm) /
+                   (rm.rows ? (long long)c.n_kv_heads * ((G * s->max_rows + 63) / 64)
+                            : (long long)rm.nb * c.n_kv_heads * rowgroups);  // splits that still fit one wave
+  if (want < 1) want = 1;
+  long long kps = ((s->cap + want - 1) / want + 63) / 64 * 64;
+  if (kps < 64) kps = 64;
+  while (want > 1 && (s->cap + kps - 1) / kps > 128) kps += 64;
+  return KeySplit{(int)((s->cap + kps - 1) / kps), (int)kps};
+}
+
+// Forwards of at most TC_CHAIN_ROWS rows: five launches per layer.  Ids are s->row_ids, or (draft_tokens
+// given) those of a verify step.
+bool use_chain(const ssd_model* m, const ssd_streams* s, RowMap rm) {
+  const int M = row_count(rm);
+  if (!m->tc.enabled || !s->ch_ssq_a || rm.rows || M > TC_CHAIN_ROWS || M > s->tc_rows) return false;
+  return s->paged || (s->path == 0 && !use_fast(m, s, rm));
+}
+
+int forward_chain(const ssd_model* m, ssd_streams* s, RowMap rm, const int32_t* draft_tokens, float* logits_out,
+                  cudaStream_t st) {
+  const ssd_model_config& c = m->cfg;
+  const int M = row_count(rm), d = c.d_model, hd = c.head_dim, n_sm = m->tc.n_sm;
+  const int qd = c.n_q_heads * hd, nq = qd + 2 * c.n_kv_heads * hd, F = c.d_ffn;
+  if (s->paged)  // every stream of this forward owns pages for the rows it is about to append
+    launch_page_ensure(s->len, rm, s->page_table, s->pages_used, s->free_stack, s->free_top, s->max_pages,
+                       s->status, st);
+  SSD_CUDA(launch_chain_embed((const bf16*)m->embed, c.vocab_out + c.vocab_text, d, draft_tokens ? nullptr : s->row_ids,
+                              s->pending, draft_tokens, s->len, rm, (const bf16*)m->layers[0].norm1, m->inv_freq, hd / 2,
+                              s->h, s->tc_xa, s->ch_ssq_a, s->rope_cs, s->status, st));
+  // how the operands are arranged: by the rows that a CTA of their consumer takes
+  const ActLay lay_qkv = tc_act_lay(chain_chunk_rows(M, d, false), d), lay_o = tc_act_lay(chain_chunk_rows(M, qd, false), qd);
+  const ActLay lay_gu = tc_act_lay(tc_round16(M), d), lay_d = tc_act_lay(tc_round16(M), F);
+  ChainGemm g{};
+  g.M = M;
+  g.inv_d = 1.0f / (float)d;
+  g.eps = c.rms_eps;
+  g.status = s->status;
+  g.h = s->h;
+  g.rope_cs = s->rope_cs;
+  g.qrot = s->qrot;
+  g.len = s->len;
+  g.rm = rm;
+  g.cap = s->cap;
+  g.Hq = c.n_q_heads;
+  g.Hkv = c.n_kv_heads;
+  g.hd_log2 = hd == 32 ? 5 : hd == 64 ? 6 : 7;
+  g.max_pages = s->max_pages;
+  g.page_table = s->page_table;
+  g.qscale = 1.0f / sqrtf((float)hd);
+  int n_ssq_a = 1;  // shares of the sums of squares: the embedding's, then the down projection's slabs
+  const int n_ssq_b = chain_split(d, qd, M, n_sm, false).clusters;
+  for (int l = 0; l < c.n_layers; ++l) {
+    const LayerW& w = m->layers[l];
+    const ssd_tc_layer& t = m->tc.layers[l];
+    g.kv_layer = (bf16*)(s->kv + (size_t)l * s->kv_layer_elems * s->el);
+    g.w = t.c_qkv; g.a = s->tc_xa; g.n_rows = nq; g.ssq_in = s->ch_ssq_a; g.n_ssq_in = n_ssq_a; g.bias = (const bf16*)w.b_qkv;
+    SSD_CUDA(launch_tc_chain(g, CHAIN_QKV, d, false, n_sm, st));
+    if (!logits_out && l + 1 == c.n_layers) break;  // only the cache is wanted: nothing reads what follows
+    if (s->attn_kernel == 0) {
+      SSD_CUDA(launch_tc_attention_chain(s->qrot, g.kv_layer, s->len, rm, s->cap, c.n_q_heads, c.n_kv_heads, hd, n_sm,
+                                         s->page_table, s->max_pages, s->tc_xattn, lay_o, s->status, st));
+    } else {
+      const KeySplit ks = key_split(m, s, rm);
+      SSD_CUDA(launch_tc_attention(s->qrot, g.kv_layer, s->len, rm, s->cap, c.n_q_heads, c.n_kv_heads, hd, s->part, ks.n,
+                                   ks.keys, s->tc_xattn, lay_o, s->page_table, s->max_pages, s->attn_kernel, s->status, st));
+    }
+    g.w = t.c_o; g.a = s->tc_xattn; g.n_rows = d; g.ssq_in = nullptr; g.gain = (const bf16*)w.norm2;
+    g.act_out = s->tc_xa; g.lay_out = lay_gu; g.ssq_out = s->ch_ssq_b;
+    SSD_CUDA(launch_tc_chain(g, CHAIN_RESIDUAL, qd, false, n_sm, st));
+    g.w = t.c_gu; g.a = s->tc_xa; g.n_rows = 2 * F; g.ssq_in = s->ch_ssq_b; g.n_ssq_in = n_ssq_b;
+    g.act_out = s->tc_xact; g.lay_out = lay_d;
+    SSD_CUDA(launch_tc_chain(g, CHAIN_SWIGLU, d, true, n_sm, st));
+    g.w = t.c_d; g.a = s->tc_xact; g.n_rows = d; g.ssq_in = nullptr;
+    g.gain = (const bf16*)(l + 1 < c.n_layers ? m->layers[l + 1].norm1 : m->norm_f);
+    g.act_out = s->tc_xa; g.lay_out = lay_qkv; g.ssq_out = s->ch_ssq_a;
+    SSD_CUDA(launch_tc_chain(g, CHAIN_RESIDUAL, F, true, n_sm, st));
+    n_ssq_a = chain_split(d, F, M, n_sm, true).clusters;
+  }
+  if (logits_out) {
+    g.w = m->tc.c_head; g.a = s->tc_xa; g.n_rows = c.vocab_out; g.ssq_in = s->ch_ssq_a; g.n_ssq_in = n_ssq_a;
+    g.out = logits_out;
+    SSD_CUDA(launch_tc_chain(g, CHAIN_LOGITS, d, false, n_sm, st));
+  }
+  SSD_CUDA(cudaGetLastError());
+  return SSD_OK;
+}
+
 int forward_tc(const ssd_model* m, ssd_streams* s, RowMap rm, float* logits_out, cudaStream_t st,
                const PrefillSegs* segs = nullptr) {
   const ssd_model_config& c = m->cfg;
@@ -361,18 +468,8 @@ int forward_tc(const ssd_model* m, ssd_streams* s, RowMap rm, float* logits_out,
     return seg ? tc_ksplit(rows, K, TC_PREFILL_CHUNK, n_sm) : pairs ? tc_prefill_groups(rows, M, (K + 63) / 64, n_sm) : tc_ksplit(rows, K, M, n_sm);
   };
   const int ks_qkv = slices(nq, d), ks_o = slices(d, qd), ks_d = slices(d, F);
-  // key splits of the attention: whole 64-key tiles, and no more CTAs in all than the SMs hold
-  // at once (a second, partly filled wave would cost as much as the first)
-  const int G = c.n_q_heads / c.n_kv_heads, rowgroups = (G * rm.R + 63) / 64;
   const int Mc = pairs ? tc_prefill_chunks(M).rows : tc_chunks(M).rows;
-  long long want = ((long long)tc_attention_ctas_per_sm(c.head_dim) * n_sm) /
-                   (seg ? (long long)c.n_kv_heads * ((G * s->max_rows + 63) / 64)
-                        : (long long)rm.nb * c.n_kv_heads * rowgroups);  // splits that still fit one wave
-  if (want < 1) want = 1;
-  long long kps = ((s->cap + want - 1) / want + 63) / 64 * 64;
-  if (kps < 64) kps = 64;
-  while (want > 1 && (s->cap + kps - 1) / kps > 128) kps += 64;  // the merge kernel's table of splits
-  const int nsplit = (int)((s->cap + kps - 1) / kps);
+  const KeySplit ks = key_split(m, s, rm);
   if (M > s->tc_rows) return SSD_ERR_BAD_PARAM;
   if (s->paged && segs)
     launch_page_ensure_segs(s->len, *segs, s->page_table, s->pages_used, s->free_stack, s->free_top, s->max_pages,
@@ -410,7 +507,7 @@ int forward_tc(const ssd_model* m, ssd_streams* s, RowMap rm, float* logits_out,
                        s->status, st);
     if (!logits_out && l + 1 == c.n_layers) break;  // only the cache is wanted: nothing reads what follows
     SSD_CUDA(launch_tc_attention(s->qrot, kv_layer, s->len, rm, s->cap, c.n_q_heads, c.n_kv_heads, c.head_dim,
-                                 s->part, nsplit, (int)kps, s->tc_xattn, lay(qd), s->page_table, s->max_pages, s->attn_kernel,
+                                 s->part, ks.n, ks.keys, s->tc_xattn, lay(qd), s->page_table, s->max_pages, s->attn_kernel,
                                  s->status, st));
     g.w = t.w_o; g.a = s->tc_xattn; g.n_rows = d; g.K = qd; g.ksplit = ks_o;
     SSD_CUDA(gemm(g, in_o, PF_EPI_RESIDUAL, nullptr, s->h));
@@ -434,6 +531,7 @@ int forward_tc(const ssd_model* m, ssd_streams* s, RowMap rm, float* logits_out,
 }
 
 int forward(const ssd_model* m, ssd_streams* s, RowMap rm, float* logits_out, cudaStream_t st) {
+  if (use_chain(m, s, rm)) return forward_chain(m, s, rm, nullptr, logits_out, st);
   if (s->paged) return forward_tc(m, s, rm, logits_out, st);
   if (use_fast(m, s, rm)) return forward_fast(m, s, rm, s->row_ids, nullptr, logits_out, st);
   if (use_tc(m, s, rm)) return forward_tc(m, s, rm, logits_out, st);
@@ -693,6 +791,11 @@ int ssd_model_create(const ssd_model_config* cfg, const void* host_weights, size
       if (e == cudaSuccess) e = tc_pack_weights((const bf16*)src, rows, K, (uint8_t*)(A + dst_off), 0);
       return (const uint8_t*)(A + dst_off);
     };
+    // and a fourth, in groups of 8 rows that a slab of any height can be cut from (tc_chain.cu)
+    auto pack_groups = [&](const void* src, int rows, int K, size_t dst_off, int hd_log2 = 0) {
+      if (e == cudaSuccess) e = chain_pack_weights((const bf16*)src, rows, K, hd_log2, (uint8_t*)(A + dst_off), 0);
+      return (const uint8_t*)(A + dst_off);
+    };
     for (int l = 0; l < c.n_layers; ++l) {
       const LayerW& w = m->layers[l];
       const LayerOff& o = p.tc_layers[l];
@@ -700,8 +803,15 @@ int ssd_model_create(const ssd_model_config* cfg, const void* host_weights, size
       t.layers[l].w_o = pack(w.w_o, (int)d, (int)qd, o.w_o);
       t.layers[l].w_gu = pack(w.w_gu, (int)(2 * F), (int)d, o.w_gu);
       t.layers[l].w_d = pack(w.w_d, (int)d, (int)F, o.w_d);
+      const LayerOff& co = p.ch_layers[l];
+      t.layers[l].c_qkv = pack_groups(w.w_qkv, (int)(qd + 2 * kvd), (int)d, co.w_qkv,
+                                      c.head_dim == 32 ? 5 : c.head_dim == 64 ? 6 : 7);
+      t.layers[l].c_o = pack_groups(w.w_o, (int)d, (int)qd, co.w_o);
+      t.layers[l].c_gu = pack_groups(w.w_gu, (int)(2 * F), (int)d, co.w_gu);
+      t.layers[l].c_d = pack_groups(w.w_d, (int)d, (int)F, co.w_d);
     }
     t.head = pack(m->head, c.vocab_out, (int)d, p.tc_head);
+    t.c_head = pack_groups(m->head, c.vocab_out, (int)d, p.ch_head);
     t.enabled = e == cudaSuccess;
   }
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -927,6 +1037,8 @@ int streams_create_impl(const ssd_model* m, int32_t batch, int32_t capacity_toke
   s->attn_part = p.attn_part ? (float*)(W + p.attn_part) : nullptr;
   s->attn_cnt = p.attn_part ? (uint32_t*)(W + p.attn_cnt) : nullptr;
   s->key_split = capacity_tokens >= KEYSPLIT_MIN_CAPACITY ? 1 : 0;
+  s->ch_ssq_a = p.tc_part ? (float*)(W + p.ch_ssq_a) : nullptr;
+  s->ch_ssq_b = p.tc_part ? (float*)(W + p.ch_ssq_b) : nullptr;
   s->tc_rowmap = p.tc_part ? (int2*)(W + p.tc_rowmap) : nullptr;
   s->tc_tiles = p.tc_part ? (int4*)(W + p.tc_tiles) : nullptr;
   s->tc_xa = p.tc_part ? (uint8_t*)(W + p.tc_xa) : nullptr;
@@ -1012,6 +1124,7 @@ int ssd_forward(ssd_model* model, ssd_streams* s, const int32_t* dev_draft_token
   cudaStream_t st = (cudaStream_t)stream;
   const RowMap rm{0, s->B, gamma + 1};
   if (use_fast(model, s, rm)) return forward_fast(model, s, rm, nullptr, dev_draft_tokens, dev_logits, st);
+  if (use_chain(model, s, rm)) return forward_chain(model, s, rm, dev_draft_tokens, dev_logits, st);
   launch_gather_verify_ids(s->pending, dev_draft_tokens, gamma, s->B, s->row_ids, st);
   return forward(model, s, rm, dev_logits, st);
 }
@@ -1186,6 +1299,8 @@ int verify_impl(ssd_model* target, ssd_streams* s, const int32_t* dev_draft_toke
   int rc;
   if (use_fast(target, s, rm)) {
     rc = forward_fast(target, s, rm, nullptr, dev_draft_tokens, logits, st);
+  } else if (use_chain(target, s, rm)) {
+    rc = forward_chain(target, s, rm, dev_draft_tokens, logits, st);
   } else {
     launch_gather_verify_ids(s->pending, dev_draft_tokens, gamma, s->B, s->row_ids, st);
     rc = forward(target, s, rm, logits, st);

@@ -108,11 +108,12 @@ struct ssd_fast_model {
 // Device-side view of the weights packed for the tensor-core projections of batched forwards (tc.h).
 struct ssd_tc_layer {
   const uint8_t *w_qkv, *w_o, *w_gu, *w_d;
+  const uint8_t *c_qkv, *c_o, *c_gu, *c_d;  // groups of 8 rows (tc_chain.cu)
 };
 struct ssd_tc_model {
   bool enabled = false;
   std::vector<ssd_tc_layer> layers;
-  const uint8_t* head = nullptr;
+  const uint8_t *head = nullptr, *c_head = nullptr;
   int n_sm = 148;  // SMs of the device the model was created on: sizes the K splits
 };
 
@@ -158,6 +159,7 @@ struct ssd_streams {
   int32_t *page_table, *pages_used, *free_stack, *free_top;
   // batched tensor-core forward: packed operands (inputs of QKV / gate-up / head, of O, of down)
   // and the partial sums of the K-split projections
+  float *ch_ssq_a, *ch_ssq_b;  // shares of the rows' sums of squares (tc_chain.cu)
   int2* tc_rowmap;  // prefill chunks: (stream, r) of every row, and the attention's tiles
   int4* tc_tiles;
   uint8_t *tc_xa, *tc_xattn, *tc_xact;

@@ -228,6 +228,57 @@ cudaError_t tc_pack_weights(const bf16* w_rowmajor, int n_rows, int K, uint8_t* 
 cudaError_t tc_unpack_weights(const uint8_t* packed, int n_rows, int K, bf16* w_rowmajor, cudaStream_t st);
 cudaError_t launch_tc_gemm(const TcGemm& g, cudaStream_t st);
 
+// tc_chain.cu: the projections of a forward of at most TC_CHAIN_ROWS rows with what sits between
+// them (norms, bias, rotary embedding, cache append, residual, SwiGLU) in their epilogues.
+constexpr int TC_CHAIN_ROWS = 128;
+enum ChainEpilogue { CHAIN_QKV = 0, CHAIN_RESIDUAL = 1, CHAIN_SWIGLU = 2, CHAIN_LOGITS = 3 };
+struct ChainGemm {
+  const uint8_t *w, *a;    // weights in groups of 8 rows (chain_pack_weights), packed activations (tc_act_lay)
+  int n_rows, M, cluster;  // cluster: set by the launcher
+  // 1/rms of the input rows: their sums of squares in n_ssq_in shares [n_ssq_in][Mpad] (null: no scaling)
+  const float* ssq_in;
+  int n_ssq_in;
+  float inv_d, eps;
+  int32_t* status;
+  // residual: h [M][n_rows]; act_out = operand of h * gain; ssq_out [slabs][Mpad].  SwiGLU: act_out
+  float* h;
+  const bf16* gain;
+  uint8_t* act_out;
+  ActLay lay_out;
+  float* ssq_out;
+  float* out;              // logits [M][n_rows]
+  // QKV
+  const bf16* bias;
+  const float* rope_cs;
+  float* qrot;
+  bf16* kv_layer;
+  const int32_t* len;
+  RowMap rm;
+  int cap, Hq, Hkv, hd_log2, max_pages;
+  const int32_t* page_table;
+  float qscale;
+};
+struct ChainSplit {
+  int cluster, clusters, tsplit;  // CTAs that split K, slabs, CTAs that split the token rows
+};
+inline bool chain_long(int K) { return K > 2048; }
+inline size_t chain_weight_bytes(int n_rows, int K) { return (size_t)((n_rows + 7) / 8) * ((K + 15) / 16) * 256; }
+// hd_log2: rows of the QKV projection, whose rotary partners become neighbours; 0: any other.
+cudaError_t chain_pack_weights(const bf16* w_rowmajor, int n_rows, int K, int hd_log2, uint8_t* packed, cudaStream_t st);
+// whole: a projection whose CTAs take all token rows whatever their number (gate/up and down).  Its operand
+// is arranged in the chunks of rows that its CTAs take.
+ChainSplit chain_split(int n_rows, int K, int M, int n_sm, bool whole);
+inline int chain_chunk_rows(int M, int K, bool whole) {
+  return whole || chain_long(K) || M <= 48 ? tc_round16(M) : tc_round16((M + 1) / 2);
+}
+cudaError_t launch_tc_chain(const ChainGemm& g, int epi, int K, bool whole, int n_sm, cudaStream_t st);
+// Rows entering the chain: ids given (row_ids) or a verify step's (each stream's pending token, then
+// its draft); embedding to h, operand and sums of squares of the first norm, rotary table.
+cudaError_t launch_chain_embed(const bf16* table, int vocab_in, int d, const int32_t* row_ids, const int32_t* pending,
+                               const int32_t* draft, const int32_t* len, RowMap rm, const bf16* gain,
+                               const double* inv_freq, int half, float* h, uint8_t* apack, float* ssq, float* cs,
+                               int32_t* status, cudaStream_t st);
+
 // tc_rows.cu
 // h[m, :] += sum of `nsplit` partial projections (part may be null); then the RMS norm of the row
 // times `gain`, written as a packed operand (hi + lo) of d columns.  h_in may differ from h (the
@@ -263,6 +314,10 @@ cudaError_t launch_tc_attention(const float* qrot, const bf16* kv_layer, const i
                                 int keys_per_split, uint8_t* apack_out, ActLay lay,
                                 const int32_t* page_table, int max_pages, int which_kernel, int32_t* status,
                                 cudaStream_t st);
+// tc_attention_chain.cu: the attention of a chain forward (uniform rows per stream), splits merged.
+cudaError_t launch_tc_attention_chain(const float* qrot, const bf16* kv_layer, const int32_t* len, RowMap rm, int cap,
+                                      int Hq, int Hkv, int hd, int n_sm, const int32_t* page_table, int max_pages,
+                                      uint8_t* apack, ActLay lay, int32_t* status, cudaStream_t st);
 int tc_attention_ctas_per_sm(int hd);  // CTAs of the attention kernel an SM holds at once
 // tc_attention5.cu: the same partial results (one per row, head and key split) on tcgen05 tensor
 // cores, for head sizes 64 and 128.  It costs less per key and more per CTA than the warp-level
