@@ -9,6 +9,7 @@
 #include <math_constants.h>
 
 #include "kernels.h"
+#include "tc.h"
 
 namespace ssd {
 
@@ -19,6 +20,7 @@ __global__ void __launch_bounds__(ATTN_WARPS * 32)
 attn_split_kernel(const float* __restrict__ qrot, const T* __restrict__ kv_layer,
                   const int32_t* __restrict__ len, RowMap rm, int cap, int Hq, int Hkv,
                   float* __restrict__ part, int nsplit_max) {
+  tc_pdl_enter();
   constexpr int NI = HD / 32;
   constexpr int KP = HD + 1;  // padded key row: lane = key reads are conflict-free
   extern __shared__ __align__(16) float smem[];
@@ -100,6 +102,7 @@ attn_split_kernel(const float* __restrict__ qrot, const T* __restrict__ kv_layer
 template <typename T, int HD>
 __global__ void attn_merge_kernel(const float* __restrict__ part, const int32_t* __restrict__ len,
                                   RowMap rm, int cap, int Hq, int nsplit_max, float* __restrict__ out) {
+  tc_pdl_enter();
   const int h = blockIdx.x, m = blockIdx.y;
   const int bi = m / rm.R, b = rm.b0 + bi;
   const int total = min(len[b] + rm.R, cap);
@@ -134,12 +137,12 @@ static cudaError_t launch_t(const float* qrot, const void* kv_layer, const int32
     if (e != cudaSuccess) return e;
   }
   dim3 grid(nsplit_max, Hkv, rm.nb);
-  kern<<<grid, ATTN_WARPS * 32, smem, st>>>(qrot, (const T*)kv_layer, len, rm, cap, Hq, Hkv, part,
-                                            nsplit_max);
+  tc_launch_pdl(kern, grid, dim3(ATTN_WARPS * 32), smem, st, qrot, (const T*)kv_layer, len, rm, cap, Hq, Hkv, part,
+                nsplit_max);
   count_launch();
   dim3 mg(Hq, rm.nb * rm.R);
-  attn_merge_kernel<T, HD><<<mg, HD < 64 ? 32 : 64, 0, st>>>(part, len, rm, cap, Hq, nsplit_max,
-                                                             out);
+  tc_launch_pdl(attn_merge_kernel<T, HD>, dim3(mg), dim3(HD < 64 ? 32 : 64), 0, st, part, len, rm, cap, Hq,
+                nsplit_max, out);
   count_launch();
   return cudaGetLastError();
 }

@@ -4,6 +4,7 @@
 #include <atomic>
 
 #include "kernels.h"
+#include "tc.h"
 
 namespace ssd {
 
@@ -15,6 +16,7 @@ uint64_t launch_count() { return g_launches.load(std::memory_order_relaxed); }
 __global__ void gather_verify_ids_kernel(const int32_t* __restrict__ pending,
                                          const int32_t* __restrict__ draft, int gamma, int B,
                                          int32_t* __restrict__ row_ids) {
+  tc_pdl_enter();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   int R = gamma + 1;
   if (i >= B * R) return;
@@ -25,8 +27,8 @@ __global__ void gather_verify_ids_kernel(const int32_t* __restrict__ pending,
 void launch_gather_verify_ids(const int32_t* pending, const int32_t* draft_tokens, int gamma,
                               int B, int32_t* row_ids, cudaStream_t st) {
   int n = B * (gamma + 1);
-  gather_verify_ids_kernel<<<(n + 127) / 128, 128, 0, st>>>(pending, draft_tokens, gamma, B,
-                                                            row_ids);
+  tc_launch_pdl(gather_verify_ids_kernel, dim3((n + 127) / 128), dim3(128), 0, st, pending, draft_tokens, gamma, B,
+                row_ids);
   count_launch();
 }
 
@@ -34,6 +36,7 @@ template <typename T>
 __global__ void embed_kernel(const T* __restrict__ table, int vocab_in, int d,
                              const int32_t* __restrict__ row_ids, float* __restrict__ h,
                              int32_t* status) {
+  tc_pdl_enter();
   int m = blockIdx.x;
   int id = row_ids[m];
   if (id < 0 || id >= vocab_in) {
@@ -47,9 +50,10 @@ __global__ void embed_kernel(const T* __restrict__ table, int vocab_in, int d,
 void launch_embed(int dtype, const void* table, int vocab_in, int d, const int32_t* row_ids, int M,
                   float* h, int32_t* status, cudaStream_t st) {
   if (dtype == 0)
-    embed_kernel<float><<<M, 128, 0, st>>>((const float*)table, vocab_in, d, row_ids, h, status);
+    tc_launch_pdl(embed_kernel<float>, dim3(M), dim3(128), 0, st, (const float*)table, vocab_in, d, row_ids, h,
+                  status);
   else
-    embed_kernel<bf16><<<M, 128, 0, st>>>((const bf16*)table, vocab_in, d, row_ids, h, status);
+    tc_launch_pdl(embed_kernel<bf16>, dim3(M), dim3(128), 0, st, (const bf16*)table, vocab_in, d, row_ids, h, status);
   count_launch();
 }
 
@@ -57,6 +61,7 @@ void launch_embed(int dtype, const void* table, int vocab_in, int d, const int32
 __global__ void rope_table_kernel(const int32_t* __restrict__ len, RowMap rm,
                                   const double* __restrict__ inv_freq, int half,
                                   float* __restrict__ cs) {
+  tc_pdl_enter();
   int m = blockIdx.x;
   const int2 br = row_at(rm, m);
   double pos = (double)(len[br.x] + br.y);
@@ -70,13 +75,14 @@ __global__ void rope_table_kernel(const int32_t* __restrict__ len, RowMap rm,
 
 void launch_rope_table(const int32_t* len, RowMap rm, const double* inv_freq, int half, float* cs,
                        cudaStream_t st) {
-  rope_table_kernel<<<row_count(rm), 64, 0, st>>>(len, rm, inv_freq, half, cs);
+  tc_launch_pdl(rope_table_kernel, dim3(row_count(rm)), dim3(64), 0, st, len, rm, inv_freq, half, cs);
   count_launch();
 }
 
 template <typename T>
 __global__ void rmsnorm_kernel(const float* __restrict__ h, const T* __restrict__ gain,
                                float* __restrict__ out, int d, float eps) {
+  tc_pdl_enter();
   __shared__ float red[32];
   int m = blockIdx.x;
   const float* x = h + (size_t)m * d;
@@ -99,9 +105,9 @@ __global__ void rmsnorm_kernel(const float* __restrict__ h, const T* __restrict_
 void launch_rmsnorm(int dtype, const float* h, const void* gain, float* out, int M, int d, float eps,
                     cudaStream_t st) {
   if (dtype == 0)
-    rmsnorm_kernel<float><<<M, 256, 0, st>>>(h, (const float*)gain, out, d, eps);
+    tc_launch_pdl(rmsnorm_kernel<float>, dim3(M), dim3(256), 0, st, h, (const float*)gain, out, d, eps);
   else
-    rmsnorm_kernel<bf16><<<M, 256, 0, st>>>(h, (const bf16*)gain, out, d, eps);
+    tc_launch_pdl(rmsnorm_kernel<bf16>, dim3(M), dim3(256), 0, st, h, (const bf16*)gain, out, d, eps);
   count_launch();
 }
 
@@ -113,6 +119,7 @@ __global__ void qkv_post_kernel(const float* __restrict__ qkv, const float* __re
                                 float* __restrict__ qrot, T* __restrict__ kv_layer,
                                 const int32_t* __restrict__ len, RowMap rm, int cap, int Hq,
                                 int Hkv, int hd, float scale, int32_t* status) {
+  tc_pdl_enter();
   int m = blockIdx.x;
   int bi = m / rm.R, r = m % rm.R, b = rm.b0 + bi;
   int pos = len[b] + r;
@@ -154,11 +161,11 @@ void launch_qkv_post(int dtype, const float* qkv, const float* cs, float* qrot, 
   float scale = 1.0f / sqrtf((float)hd);
   int M = rm.nb * rm.R;
   if (dtype == 0)
-    qkv_post_kernel<float><<<M, 128, 0, st>>>(qkv, cs, qrot, (float*)kv_layer, len, rm, cap, Hq,
-                                              Hkv, hd, scale, status);
+    tc_launch_pdl(qkv_post_kernel<float>, dim3(M), dim3(128), 0, st, qkv, cs, qrot, (float*)kv_layer, len, rm, cap,
+                  Hq, Hkv, hd, scale, status);
   else
-    qkv_post_kernel<bf16><<<M, 128, 0, st>>>(qkv, cs, qrot, (bf16*)kv_layer, len, rm, cap, Hq, Hkv,
-                                             hd, scale, status);
+    tc_launch_pdl(qkv_post_kernel<bf16>, dim3(M), dim3(128), 0, st, qkv, cs, qrot, (bf16*)kv_layer, len, rm, cap, Hq,
+                  Hkv, hd, scale, status);
   count_launch();
 }
 
@@ -179,6 +186,7 @@ void launch_advance_len(int32_t* len, int32_t* pending, int b, int add, const in
 __global__ void prefill_stage_kernel(const __grid_constant__ PrefillSegs P, const int32_t* __restrict__ ids,
                                      int32_t* __restrict__ row_ids, int2* __restrict__ rows,
                                      int4* __restrict__ tiles) {
+  tc_pdl_enter();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < P.n_rows) {
     int q = 0;
@@ -199,13 +207,15 @@ __global__ void prefill_stage_kernel(const __grid_constant__ PrefillSegs P, cons
 
 void launch_prefill_stage(const PrefillSegs& segs, const int32_t* ids, int32_t* row_ids, int2* rows, int4* tiles,
                           cudaStream_t st) {
-  prefill_stage_kernel<<<(segs.n_rows + 127) / 128, 128, 0, st>>>(segs, ids, row_ids, rows, tiles);
+  tc_launch_pdl(prefill_stage_kernel, dim3((segs.n_rows + 127) / 128), dim3(128), 0, st, segs, ids, row_ids, rows,
+                tiles);
   count_launch();
 }
 
 // The chunk's rows are in the cache: lengths grow, prompts that end here leave their last id pending.
 __global__ void prefill_advance_kernel(const __grid_constant__ PrefillSegs P, const int32_t* __restrict__ ids,
                                        int32_t* len, int32_t* pending) {
+  tc_pdl_enter();
   const int q = threadIdx.x;
   if (q >= P.n) return;
   len[P.s[q].stream] += P.s[q].count;
@@ -214,13 +224,14 @@ __global__ void prefill_advance_kernel(const __grid_constant__ PrefillSegs P, co
 
 void launch_prefill_advance(const PrefillSegs& segs, const int32_t* ids, int32_t* len, int32_t* pending,
                             cudaStream_t st) {
-  prefill_advance_kernel<<<1, PREFILL_SEGS, 0, st>>>(segs, ids, len, pending);
+  tc_launch_pdl(prefill_advance_kernel, dim3(1), dim3(PREFILL_SEGS), 0, st, segs, ids, len, pending);
   count_launch();
 }
 
 // O(1) rollback from device arrays: len[b] = src_len[b] (clamped to the capacity).
 __global__ void kv_restore_kernel(int32_t* len, int32_t* pending, const int32_t* src_len,
                                   const int32_t* src_pending, int B, int cap) {
+  tc_pdl_enter();
   int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
   len[b] = min(max(src_len[b], 0), cap);
@@ -229,12 +240,14 @@ __global__ void kv_restore_kernel(int32_t* len, int32_t* pending, const int32_t*
 
 void launch_kv_restore(int32_t* len, int32_t* pending, const int32_t* src_len,
                        const int32_t* src_pending, int B, int cap, cudaStream_t st) {
-  kv_restore_kernel<<<(B + 127) / 128, 128, 0, st>>>(len, pending, src_len, src_pending, B, cap);
+  tc_launch_pdl(kv_restore_kernel, dim3((B + 127) / 128), dim3(128), 0, st, len, pending, src_len, src_pending, B,
+                cap);
   count_launch();
 }
 
 // Draft bookkeeping: every stream's committed length grows by `add`.
 __global__ void advance_all_kernel(int32_t* len, int B, int add, int cap, int32_t* status) {
+  tc_pdl_enter();
   int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
   int nl = len[b] + add;
@@ -246,7 +259,7 @@ __global__ void advance_all_kernel(int32_t* len, int B, int add, int cap, int32_
 }
 
 void launch_advance_all(int32_t* len, int B, int add, int cap, int32_t* status, cudaStream_t st) {
-  advance_all_kernel<<<(B + 127) / 128, 128, 0, st>>>(len, B, add, cap, status);
+  tc_launch_pdl(advance_all_kernel, dim3((B + 127) / 128), dim3(128), 0, st, len, B, add, cap, status);
   count_launch();
 }
 

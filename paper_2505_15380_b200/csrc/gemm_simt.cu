@@ -5,6 +5,7 @@
 // shuffles.  The projections of the verify forward (Sec. 3.1 decoder) are skinny
 // (M = B * (gamma+1) rows), so the weights dominate the bytes.
 #include "kernels.h"
+#include "tc.h"
 
 namespace ssd {
 
@@ -16,6 +17,7 @@ template <typename T, int EPI, int KS>
 __global__ void __launch_bounds__(GEMM_WARPS * 32)
 gemm_simt_kernel(const float* __restrict__ A, int lda, const T* __restrict__ W,
                  const T* __restrict__ bias, float* __restrict__ C, int ldc, int M, int N, int K) {
+  tc_pdl_enter();
   // KS warps share one pair of columns, each taking every KS-th 256-element slice of K; the
   // CTA covers NG = GEMM_WARPS / KS column pairs.
   constexpr int NG = GEMM_WARPS / KS;
@@ -133,7 +135,7 @@ static cudaError_t launch_ks(const float* A, int lda, const void* W, const void*
   }
   constexpr int cols = (GEMM_WARPS / KS) * 2;
   dim3 grid((N + cols - 1) / cols, (M + GEMM_MT - 1) / GEMM_MT);
-  kern<<<grid, GEMM_WARPS * 32, smem, st>>>(A, lda, (const T*)W, (const T*)bias, C, ldc, M, N, K);
+  tc_launch_pdl(kern, grid, dim3(GEMM_WARPS * 32), smem, st, A, lda, (const T*)W, (const T*)bias, C, ldc, M, N, K);
   count_launch();
   return cudaGetLastError();
 }

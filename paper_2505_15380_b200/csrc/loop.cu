@@ -2,6 +2,7 @@
 // trip): which uniforms an iteration consumes, and what "append to T_in" means for the draft
 // model's cache and for the emitted token stream.
 #include "kernels.h"
+#include "tc.h"
 
 namespace ssd {
 
@@ -11,6 +12,7 @@ namespace ssd {
 __global__ void loop_stage_uniforms_kernel(const float* __restrict__ pool, int n_rows,
                                            const int32_t* __restrict__ iteration, int B, int gamma,
                                            float* __restrict__ draft_uni, float* __restrict__ verify_uni) {
+  tc_pdl_enter();
   const int per = gamma + 2 * (gamma + 1);
   const int it = ((*iteration % n_rows) + n_rows) % n_rows;
   const float* row = pool + (size_t)it * B * per;
@@ -24,8 +26,8 @@ __global__ void loop_stage_uniforms_kernel(const float* __restrict__ pool, int n
 void launch_loop_stage_uniforms(const float* pool, int n_rows, const int32_t* iteration, int B, int gamma,
                                 float* draft_uni, float* verify_uni, cudaStream_t st) {
   const int n = B * (gamma + 2 * (gamma + 1));
-  loop_stage_uniforms_kernel<<<(n + 255) / 256, 256, 0, st>>>(pool, n_rows, iteration, B, gamma, draft_uni,
-                                                             verify_uni);
+  tc_launch_pdl(loop_stage_uniforms_kernel, dim3((n + 255) / 256), dim3(256), 0, st, pool, n_rows, iteration, B,
+                gamma, draft_uni, verify_uni);
   count_launch();
 }
 
@@ -43,6 +45,7 @@ __global__ void loop_finish_kernel(int32_t* draft_len, int32_t* draft_pending, i
                                    const int32_t* __restrict__ next_token, int B, int32_t* out_tokens,
                                    int out_capacity, int32_t* out_count, int32_t* accept_log, int n_rows,
                                    int32_t* iteration, int32_t* recent, int win, int32_t* status) {
+  tc_pdl_enter();
   const int it = ((*iteration % n_rows) + n_rows) % n_rows;
   for (int b = threadIdx.x; b < B; b += blockDim.x) {  // launched as one block
     int k = accepted_len[b];
@@ -84,9 +87,9 @@ void launch_loop_finish(int32_t* draft_len, int32_t* draft_pending, int cap, int
                         int32_t* out_count, int32_t* accept_log, int n_rows, int32_t* iteration,
                         int32_t* recent_tokens, int ras_window, int32_t* status, cudaStream_t st) {
   // one block: every thread reads the iteration counter before the last thread advances it
-  loop_finish_kernel<<<1, 1024, 0, st>>>(draft_len, draft_pending, cap, in_ids, draft_tokens, gamma, accepted_len,
-                                         next_token, B, out_tokens, out_capacity, out_count, accept_log, n_rows,
-                                         iteration, recent_tokens, ras_window, status);
+  tc_launch_pdl(loop_finish_kernel, dim3(1), dim3(1024), 0, st, draft_len, draft_pending, cap, in_ids, draft_tokens,
+                gamma, accepted_len, next_token, B, out_tokens, out_capacity, out_count, accept_log, n_rows,
+                iteration, recent_tokens, ras_window, status);
   count_launch();
 }
 

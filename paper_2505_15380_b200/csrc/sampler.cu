@@ -10,6 +10,7 @@
 #include <mutex>
 
 #include "kernels.h"
+#include "tc.h"
 
 namespace ssd {
 
@@ -391,6 +392,7 @@ verify_sampler_kernel(const float* __restrict__ logits, int V,
                       int gamma, float inv_t, int top_k, float top_p, float beta, Ras ras, float* row_stats,
                       int32_t* accept_flags, int32_t* counters, int32_t* __restrict__ accepted_len,
                       int32_t* __restrict__ next_token, int32_t* status) {
+  tc_pdl_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SampSmem& sm = *reinterpret_cast<SampSmem*>(smem_raw);
   float* z = reinterpret_cast<float*>(smem_raw + sizeof(SampSmem));
@@ -513,9 +515,9 @@ cudaError_t launch_verify_sampler(const float* logits, int V, const int32_t* dra
     if (e != cudaSuccess) return e;
   }
   dim3 grid(gamma + 1, B);
-  verify_sampler_kernel<<<grid, SAMP_THREADS, smem, st>>>(
-      logits, V, draft_tokens, draft_probs, uniforms, gamma, inv_temperature, top_k, top_p, beta, ras,
-      row_stats, accept_flags, counters, accepted_len, next_token, status);
+  tc_launch_pdl(verify_sampler_kernel, grid, dim3(SAMP_THREADS), smem, st, logits, V, draft_tokens, draft_probs,
+                uniforms, gamma, inv_temperature, top_k, top_p, beta, ras, row_stats, accept_flags, counters,
+                accepted_len, next_token, status);
   count_launch();
   return cudaGetLastError();
 }
@@ -527,6 +529,7 @@ draft_sampler_kernel(const float* __restrict__ logits, int ld_logits, int V,
                      const float* __restrict__ uniform, float inv_t, int top_k, float top_p,
                      int32_t* __restrict__ out_token, int tok_stride, float* __restrict__ out_prob,
                      size_t prob_stride, int32_t* pending, int32_t* status) {
+  tc_pdl_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SampSmem& sm = *reinterpret_cast<SampSmem*>(smem_raw);
   float* z = reinterpret_cast<float*>(smem_raw + sizeof(SampSmem));
@@ -571,9 +574,8 @@ cudaError_t launch_draft_sampler(const float* logits, int ld_logits, int V, cons
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  draft_sampler_kernel<<<B, SAMP_THREADS, smem, st>>>(logits, ld_logits, V, uniform,
-                                                      inv_temperature, top_k, top_p, out_token, tok_stride,
-                                                      out_prob_row, prob_stride, pending, status);
+  tc_launch_pdl(draft_sampler_kernel, dim3(B), dim3(SAMP_THREADS), smem, st, logits, ld_logits, V, uniform,
+                inv_temperature, top_k, top_p, out_token, tok_stride, out_prob_row, prob_stride, pending, status);
   count_launch();
   return cudaGetLastError();
 }
@@ -582,6 +584,7 @@ cudaError_t launch_draft_sampler(const float* logits, int ld_logits, int V, cons
 __global__ void kv_commit_kernel(int32_t* len, int32_t* pending, const int32_t* accepted_len,
                                  const int32_t* next_token, int B, int cap, int max_gamma,
                                  int32_t* status) {
+  tc_pdl_enter();
   int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
   const int k = accepted_len[b];
@@ -601,8 +604,8 @@ __global__ void kv_commit_kernel(int32_t* len, int32_t* pending, const int32_t* 
 void launch_kv_commit(int32_t* len, int32_t* pending, const int32_t* accepted_len,
                       const int32_t* next_token, int B, int cap, int max_gamma, int32_t* status,
                       cudaStream_t st) {
-  kv_commit_kernel<<<(B + 127) / 128, 128, 0, st>>>(len, pending, accepted_len, next_token, B, cap,
-                                                    max_gamma, status);
+  tc_launch_pdl(kv_commit_kernel, dim3((B + 127) / 128), dim3(128), 0, st, len, pending, accepted_len, next_token, B,
+                cap, max_gamma, status);
   count_launch();
 }
 

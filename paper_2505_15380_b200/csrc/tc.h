@@ -67,6 +67,13 @@ enum TcEpilogue {
 #ifdef __CUDACC__
 __device__ __forceinline__ void tc_pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void tc_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The same for a kernel that has nothing to do ahead of its predecessor's results.  Its own successors
+// start when it has passed the wait: whatever they do before theirs may then rely on everything
+// older than this kernel being complete.
+__device__ __forceinline__ void tc_pdl_enter() {
+  tc_pdl_wait();
+  tc_pdl_trigger();
+}
 template <typename... KArgs, typename... Args>
 inline cudaError_t tc_launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                  Args... args) {
@@ -134,7 +141,7 @@ struct ActLay {
   uint32_t chunk;  // bytes per chunk
 #ifdef __CUDACC__
   __device__ __forceinline__ uint8_t* row(uint8_t* base, int t) const {
-    const int ch = t / Mc;
+    const int ch = t < Mc ? 0 : t / Mc;
     return base + (size_t)ch * chunk + (size_t)(t - ch * Mc) * 16;
   }
   __device__ __forceinline__ size_t col(int k) const {

@@ -213,6 +213,7 @@ __device__ __forceinline__ void page_ensure_stream(const int32_t* __restrict__ l
 __global__ void page_ensure_kernel(const int32_t* __restrict__ len, RowMap rm, int32_t* page_table,
                                    int32_t* pages_used, const int32_t* __restrict__ free_stack, int32_t* free_top,
                                    int max_pages, int32_t* status) {
+  tc_pdl_enter();
   const int bi = blockIdx.x * blockDim.x + threadIdx.x;
   if (bi < rm.nb)
     page_ensure_stream(len, rm.b0 + bi, rm.R, page_table, pages_used, free_stack, free_top, max_pages, status);
@@ -224,12 +225,14 @@ __global__ void page_ensure_segs_kernel(const int32_t* __restrict__ len, const _
                                         int32_t* page_table, int32_t* pages_used,
                                         const int32_t* __restrict__ free_stack, int32_t* free_top, int max_pages,
                                         int32_t* status) {
+  tc_pdl_enter();
   for (int q = 0; q < P.n; ++q)
     page_ensure_stream(len, P.s[q].stream, P.s[q].count, page_table, pages_used, free_stack, free_top, max_pages, status);
 }
 
 __global__ void page_release_kernel(const int32_t* __restrict__ len, int B, int32_t* page_table, int32_t* pages_used,
                                     int32_t* free_stack, int32_t* free_top, int max_pages) {
+  tc_pdl_enter();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
   const int keep = (max(len[b], 0) + TC_PAGE_TOKENS - 1) / TC_PAGE_TOKENS;
@@ -248,20 +251,20 @@ __global__ void page_release_kernel(const int32_t* __restrict__ len, int B, int3
 void launch_page_ensure(const int32_t* len, RowMap rm, int32_t* page_table, int32_t* pages_used,
                         int32_t* free_stack, int32_t* free_top, int max_pages, int32_t* status,
                         cudaStream_t st) {
-  page_ensure_kernel<<<(rm.nb + 127) / 128, 128, 0, st>>>(len, rm, page_table, pages_used, free_stack, free_top,
+  tc_launch_pdl(page_ensure_kernel, dim3((rm.nb + 127) / 128), dim3(128), 0, st, len, rm, page_table, pages_used, free_stack, free_top,
                                                          max_pages, status);
   count_launch();
 }
 
 void launch_page_ensure_segs(const int32_t* len, const PrefillSegs& segs, int32_t* page_table, int32_t* pages_used,
                              int32_t* free_stack, int32_t* free_top, int max_pages, int32_t* status, cudaStream_t st) {
-  page_ensure_segs_kernel<<<1, 1, 0, st>>>(len, segs, page_table, pages_used, free_stack, free_top, max_pages, status);
+  tc_launch_pdl(page_ensure_segs_kernel, dim3(1), dim3(1), 0, st, len, segs, page_table, pages_used, free_stack, free_top, max_pages, status);
   count_launch();
 }
 
 void launch_page_release(const int32_t* len, int B, int32_t* page_table, int32_t* pages_used,
                          int32_t* free_stack, int32_t* free_top, int max_pages, cudaStream_t st) {
-  page_release_kernel<<<(B + 127) / 128, 128, 0, st>>>(len, B, page_table, pages_used, free_stack, free_top,
+  tc_launch_pdl(page_release_kernel, dim3((B + 127) / 128), dim3(128), 0, st, len, B, page_table, pages_used, free_stack, free_top,
                                                       max_pages);
   count_launch();
 }
