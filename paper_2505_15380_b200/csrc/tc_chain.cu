@@ -182,15 +182,20 @@ __global__ void __launch_bounds__(CH_THREADS) tc_chain_kernel(const __grid_const
       const uint32_t idesc = umma_idesc(2 * P.Mc);
       const uint64_t da = umma_desc(smem_u32(smem), 128u, gstride);
       const uint64_t db = umma_desc(smem_u32(smem) + stage_w, (uint32_t)P.Mc * 32u, 128u);
+      const uint32_t ahi = (uint32_t)(da >> 32), bhi = (uint32_t)(db >> 32), alo = (uint32_t)da, blo = (uint32_t)db;
       uint32_t s = 0, par = 0;
       for (int it = 0; it < n_iter; ++it) {
         if (!mbar_wait(smem_u32(&S.full[s]), par, abort)) break;
         fence_after();
         const int nk = min(P.sk, k1 - k0 - it * P.sk);
-        const uint64_t a = da + (uint64_t)((s * stage_bytes) >> 4), b = db + (uint64_t)((s * stage_bytes) >> 4);
+        const uint32_t off = (s * stage_bytes) >> 4, a = alo + off, b = blo + off, bstep = act_block >> 4;
+        if (nk == CH_SK) {  // straight-line: what the issuing thread executes is what these short instructions cost
+          umma_bf16_lo(tmem, a, ahi, b, bhi, idesc, it > 0 ? 1u : 0u);
 #pragma unroll
-        for (int j = 0; j < CH_SK; ++j)
-          if (j < nk) umma_bf16(tmem, a + (uint64_t)(j * 16), b + (uint64_t)(j * (act_block >> 4)), idesc, it > 0 || j > 0 ? 1u : 0u);
+          for (int j = 1; j < CH_SK; ++j) umma_bf16_lo(tmem, a + j * 16, ahi, b + j * bstep, bhi, idesc, 1u);
+        } else {
+          for (int j = 0; j < nk; ++j) umma_bf16_lo(tmem, a + j * 16, ahi, b + j * bstep, bhi, idesc, it > 0 || j > 0 ? 1u : 0u);
+        }
         umma_commit(smem_u32(&S.empty[s]));
         if (++s == (uint32_t)P.stages) {
           s = 0;
@@ -406,11 +411,20 @@ __global__ void __launch_bounds__(CH_THREADS) tc_chain_kernel(const __grid_const
 #pragma unroll
         for (int q = 0; q < 4; ++q) x[q] = hv[q] * rp.gain;
         store_pair4(G.lay_out, G.act_out, t0 + quad * 4, n & ~1, lane, x, ok ? valid : 0);
+        float ss[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          float ss = q < valid ? hv[q] * hv[q] : 0.f;
-          for (int o = RW >> 1; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-          if (sublane == 0 && have && q < valid) sq[(quad * 4 + q) * rw + rp.rb] = ss;
+        for (int q = 0; q < 4; ++q) ss[q] = q < valid ? hv[q] * hv[q] : 0.f;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          if (o < RW) {  // uniform
+#pragma unroll
+            for (int q = 0; q < 4; ++q) ss[q] += __shfl_xor_sync(0xffffffffu, ss[q], o);
+          }
+        }
+        if (sublane == 0 && have) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (q < valid) sq[(quad * 4 + q) * rw + rp.rb] = ss[q];
         }
       }
       __syncthreads();  // (every thread of the CTA is here)
@@ -459,8 +473,7 @@ chain_embed_kernel(const bf16* __restrict__ table, int vocab_in, int d, const in
                    ActLay lay, float* __restrict__ ssq, float* __restrict__ cs, int32_t* status) {
   __shared__ float red[8];
   const int m = blockIdx.x, tid = threadIdx.x;
-  tc_pdl_trigger();
-  tc_pdl_wait();
+  tc_pdl_enter();  // not before the wait: the attention of the first layer relies on older kernels being complete
   const int2 br = row_at(rm, m);
   int id = row_ids ? row_ids[m] : br.y == 0 ? pending[br.x] : draft[(size_t)br.x * (rm.R - 1) + br.y - 1];
   if (id < 0 || id >= vocab_in) {
@@ -590,13 +603,15 @@ cudaError_t launch_tc_chain(const ChainGemm& g, int epi, int K, bool whole, int 
   const size_t red = (size_t)cs.cluster * p.Tcp * p.rows_max * 4 * (cs.cluster > 1 ? 2 : 1);  // gathered, and pushed
   const int ks_cta = (p.KS + cs.cluster - 1) / cs.cluster;
   const size_t per_ks = (size_t)p.ng_max * 256 + (size_t)p.Mc * 64;
-  // half an SM (the next projection's CTAs then come in while this one's finish) where that holds all of
-  // a CTA's operands, else the whole of it: with two stages in flight a CTA took in 26 bytes per
-  // cycle (measured), with five 70
-  size_t budget = 112 * 1024 - sizeof(ChShared) - 128;
-  if (ks_cta * per_ks + red > budget) budget = 226 * 1024 - sizeof(ChShared) - 128;
+  // half an SM (the next kernel's CTAs then come in while this one's finish) where that holds all of a
+  // CTA's operands or three stages of at least 16 KB, else the whole of it: with two stages in flight a
+  // CTA took in 26 bytes per cycle (measured), with five 70
+  size_t budget = 111 * 1024 - sizeof(ChShared) - 128;
   p.sk = std::min(CH_SK, ks_cta);
-  while (p.sk > 2 && 4 * p.sk * per_ks + red > budget && p.sk * per_ks > 32768) p.sk = (p.sk + 1) / 2;
+  if (ks_cta * per_ks + red > budget && (3 * p.sk * per_ks + red > budget || p.sk * per_ks < 16384)) {
+    budget = 226 * 1024 - sizeof(ChShared) - 128;
+    while (p.sk > 2 && 4 * p.sk * per_ks + red > budget && p.sk * per_ks > 32768) p.sk = (p.sk + 1) / 2;
+  }
   if (2 * p.sk * per_ks + red > budget) return cudaErrorInvalidValue;
   p.stages = (int)std::min((budget - red) / (p.sk * per_ks), (size_t)CH_MAX_STAGES);
   p.stages = std::min(p.stages, (ks_cta + p.sk - 1) / p.sk);
