@@ -282,7 +282,7 @@ bool same_shape(const ssd_model_config& a, const ssd_model_config& b) {
 // rows' K/V at len + r; when logits_out is non-null also runs the final norm and the LM head.
 // The persistent kernel covers forwards of at most FAST_MAX_T rows over a bf16 model.
 bool use_fast(const ssd_model* m, const ssd_streams* s, RowMap rm) {
-  return m->fast.enabled && s->path == 0 && !s->paged && !rm.rows && rm.nb * rm.R <= FAST_MAX_T;
+  return m->fast.enabled && s->path == 0 && !s->paged && !rm.rows && rm.nb * rm.R <= (rm.nb > 1 ? 8 : FAST_MAX_T);
 }
 
 int forward_fast(const ssd_model* m, ssd_streams* s, RowMap rm, const int32_t* row_ids,

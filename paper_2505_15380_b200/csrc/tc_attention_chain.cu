@@ -14,6 +14,8 @@
 // barrier, instead of through memory to a merge kernel (one launch, one round trip and 6 us less).
 #include <math_constants.h>
 
+#include <algorithm>
+
 #include "kernels.h"
 #include "tc.h"
 #include "tc_ptx.cuh"
@@ -61,10 +63,10 @@ struct AcLay {
   static constexpr int STAGES = HD == 128 ? 2 : 3;
   static constexpr int Q_BYTES = 4 * (HD / 16) * 32 * 32;
   static constexpr int PW = HD + 4;                    // floats of a row's partial: output, max, sum, padding
-  static constexpr int PART = 2 * 64 * PW * 4;         // two halves x 64 rows
-  static constexpr int OFF_Q = STAGES * STAGE, OFF_G = OFF_Q + Q_BYTES;
+  static constexpr int PART = 2 * 70 * PW * 4;         // two halves x 64 rows, rounded up to the owners' shares
+  static constexpr int OFF_Q = STAGES * STAGE > PART ? STAGES * STAGE : PART;  // the outgoing partials take the tiles' place
+  static constexpr int OFF_G = OFF_Q + Q_BYTES;
   static constexpr int OFF_B = OFF_G + PART, TOTAL = OFF_B + 32;
-  static_assert(PART <= STAGES * STAGE, "the outgoing partials take the place of the tiles");
 };
 
 template <int HD>
@@ -261,7 +263,7 @@ tc_attn_chain_kernel(const float* __restrict__ qrot, const bf16* __restrict__ kv
   __syncthreads();  // the tiles are dead: their place takes the outgoing partials
 
   // ---- partials to the CTAs that own their rows (RPO rows each)
-  const int RPO = 64 / S, block = 2 * RPO * PW;
+  const int RPO = (64 + S - 1) / S, block = 2 * RPO * PW;
   if (active) {
 #pragma unroll
     for (int hh = 0; hh < 2; ++hh) {
@@ -282,7 +284,7 @@ tc_attn_chain_kernel(const float* __restrict__ qrot, const bf16* __restrict__ kv
     if (warp == 0 && elect_one()) {
       mbar_expect_tx(smem_u32(bar), (uint32_t)(S * block) * 4u);
       for (int i = 0; i < S; ++i) {
-        const uint32_t to = (uint32_t)((rank + i) & (S - 1));
+        const uint32_t to = (uint32_t)(rank + i < S ? rank + i : rank + i - S);
         asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                      ::"r"(map_rank(smem_u32(gath) + (uint32_t)(rank * block) * 4u, to)),
                      "r"(smem_u32(push) + to * (uint32_t)block * 4u), "r"((uint32_t)block * 4u), "r"(map_rank(smem_u32(bar), to))
@@ -298,7 +300,7 @@ tc_attn_chain_kernel(const float* __restrict__ qrot, const bf16* __restrict__ kv
   const int np = 2 * S;
   for (int rl = warp; rl < RPO; rl += AC_THREADS / 32) {
     const int i = rg * 64 + rank * RPO + rl;
-    if (i >= NQ) break;
+    if (rank * RPO + rl >= 64 || i >= NQ) break;
     const float* base = gath + (size_t)rl * PW;
     float pm = -CUDART_INF_F, pl = 0.f;
     if (lane < np) {
@@ -312,14 +314,15 @@ tc_attn_chain_kernel(const float* __restrict__ qrot, const bf16* __restrict__ kv
 #pragma unroll
     for (int c = 0; c < (HD + 63) / 64; ++c) {
       const int d = c * 64 + lane * 2;
-      float2 acc = make_float2(0.f, 0.f);
-      for (int p = 0; p < np; ++p) {  // fixed order
+      float2 acc = make_float2(0.f, 0.f), v[16];
+#pragma unroll
+      for (int p = 0; p < 16; ++p)  // all loads in flight
+        v[p] = p < np && d < HD ? *reinterpret_cast<const float2*>(base + (size_t)p * RPO * PW + d) : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int p = 0; p < 16; ++p) {  // fixed order; absent partials weigh nothing
         const float w = __shfl_sync(0xffffffffu, e, p);
-        if (d < HD) {
-          const float2 v = *reinterpret_cast<const float2*>(base + (size_t)p * RPO * PW + d);
-          acc.x = fmaf(w, v.x, acc.x);
-          acc.y = fmaf(w, v.y, acc.y);
-        }
+        acc.x = fmaf(w, v[p].x, acc.x);
+        acc.y = fmaf(w, v[p].y, acc.y);
       }
       if (d < HD) {
         uint32_t hi, lo;
@@ -339,9 +342,11 @@ cudaError_t launch_t(const float* qrot, const bf16* kv_layer, const int32_t* len
                      int n_sm, const int32_t* page_table, int max_pages, uint8_t* apack, ActLay lay, int32_t* status,
                      cudaStream_t st) {
   const int rowgroups = ((Hq / Hkv) * rm.R + 63) / 64, items = rm.nb * Hkv * rowgroups;
-  // splits: as many CTAs as fit the SMs at once, no more than there are tiles
-  int S = 1;
-  while (S < 8 && items * S * 2 <= (HD == 128 ? 1 : 2) * n_sm && S * AC_TILE < cap) S *= 2;
+  // splits: no more than there are tiles, and as many CTAs as fit the SMs at once with a margin - the CTAs of
+  // a cluster need SMs of one GPC, and 32 clusters of 8 at two CTAs per SM left one for a second wave
+  // (17.6 us; 32 clusters of 7 do not)
+  const int room = (HD == 128 ? 3 : 6) * n_sm / 4 / items;
+  const int S = std::max(1, std::min(std::min(8, room), (cap + AC_TILE - 1) / AC_TILE));
   cudaError_t e = cudaFuncSetAttribute(tc_attn_chain_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, AcLay<HD>::TOTAL);
   if (e != cudaSuccess) return e;
   e = tc_launch_pdl_cluster(tc_attn_chain_kernel<HD>, dim3(S, Hkv * rowgroups, rm.nb), dim3(AC_THREADS), S,

@@ -51,7 +51,7 @@ struct ChShared {
   unsigned long long full[CH_MAX_STAGES], empty[CH_MAX_STAGES], accum, gathered;
   uint32_t tmem_base;
   int abort;
-  alignas(16) float inv_rms[TC_CHAIN_ROWS * 4];  // of this CTA's token rows; residual epilogue: the warps' sums of squares
+  alignas(16) float inv_rms[TC_CHAIN_ROWS * 16];  // of this CTA's token rows; residual epilogue: its blocks' sums of squares
 };
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
@@ -72,6 +72,15 @@ __device__ __forceinline__ void store_quad(uint8_t* row, const ActLay& lay, int 
   *reinterpret_cast<uint2*>(e) = make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
   *reinterpret_cast<uint2*>(e + lay.part_off) =
       make_uint2(*reinterpret_cast<const uint32_t*>(&l0), *reinterpret_cast<const uint32_t*>(&l1));
+}
+// Column k of a token's row, in lanes whose neighbour (lane ^ 4) holds column k ^ 1: the even lane of the
+// pair stores both leading parts, the odd one both remainders, a word each.  All lanes take part.
+__device__ __forceinline__ void store_shared(uint8_t* row, const ActLay& lay, int k, float x, bool valid) {
+  const bf16 h = __float2bfloat16_rn(x), l = __float2bfloat16_rn(x - __bfloat162float(h));
+  const uint32_t hb = __bfloat16_as_ushort(h), lb = __bfloat16_as_ushort(l), odd = (uint32_t)k & 1u;
+  const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? hb : lb, 4);
+  if (valid)
+    *reinterpret_cast<uint32_t*>(row + lay.col(k & ~1) + (odd ? lay.part_off : 0u)) = odd ? got | (lb << 16) : hb | (got << 16);
 }
 // Token rows t .. t + 3 (t a multiple of 4, so all of one chunk) of columns k (even lanes) and k + 1 (odd
 // lanes): the lanes of a pair exchange two rows each, so that every store is a whole word.
@@ -220,71 +229,62 @@ __global__ void __launch_bounds__(CH_THREADS) tc_chain_kernel(const __grid_const
     }
   }
 
-  // ---- what this thread's first epilogue task reads from memory, while the instructions run.  Warps 2..7
-  // come first: the copying and the issuing warp have other work until now.
+  // ---- the epilogue's tasks: a warp takes a quad of token rows x a block of 8 weight rows (QKV: of 8 rotary
+  // pairs; SwiGLU: of 8 columns of its output), one element per lane: token lane % 4, row lane / 4.  So
+  // shared memory is read without conflicts, operands are stored in contiguous 16-byte rows, and the
+  // code is short: it runs once or twice per launch, and what it costs is mostly its instruction
+  // fetches (four token rows per thread, unrolled, took 2200 cycles).  What the first task reads from memory
+  // is requested while the instructions run; warps 2..7 come first, the copying and the issuing warp
+  // have other work until now.
   const int tr = rank * P.Tc, t0 = tbase + tr, nt = min(P.Tc, M - tr), n_quads = (nt + 3) >> 2;
-  const int task0 = (tid + CH_THREADS - 64) & (CH_THREADS - 1);
+  const int n_elems = EPI == CHAIN_QKV || EPI == CHAIN_SWIGLU ? rows >> 1 : rows, n_blocks = (n_elems + 7) >> 3;
+  const int n_tasks = n_quads * n_blocks, task0 = (warp + 6) & 7;
   const int hl2 = G.hd_log2, half = 1 << (hl2 - 1);
-  const size_t rows_per = G.page_table ? (size_t)TC_PAGE_TOKENS : (size_t)G.cap;
-  // QKV: weight rows 2 e and 2 e + 1 of the slab are a rotary pair (j, j + hd / 2) of head hh (chain_qkv_row)
-  struct QkvTask {
-    int quad, e, hh, j, owner[4], slot[4];
-    float bx, by;
-    float2 cs[4];
-  } qp;
-  auto load_qkv = [&](int i, QkvTask& p) {
-    const int pairs = rows >> 1;
-    p.quad = i / pairs;
-    p.e = i - p.quad * pairs;
-    const int pr = (n0 >> 1) + p.e;
-    p.hh = pr >> (hl2 - 1);
-    p.j = pr & (half - 1);
-    p.bx = __bfloat162float(G.bias[(p.hh << hl2) + p.j]);
-    p.by = __bfloat162float(G.bias[(p.hh << hl2) + p.j + half]);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int t = min(t0 + p.quad * 4 + q, G.M - 1);
-      p.cs[q] = make_float2(1.f, 0.f);
-      if (p.hh < G.Hq + G.Hkv) p.cs[q] = __ldcg(reinterpret_cast<const float2*>(G.rope_cs + ((size_t)t << hl2) + 2 * p.j));
-      if (p.hh >= G.Hq) {  // where the row's K or V lives: the stream's slice of a contiguous cache, or its page
-        const int2 br = row_at(G.rm, t);
+  struct Task {
+    int tl, t, e, blk;      // token row of this CTA, of the forward; element; its block
+    bool ok;
+    int hh, j, owner, slot; // QKV: head, rotary pair, where K or V goes
+    float2 cs, bias;
+    float h, gain;          // residual
+  } T;
+  auto load_task = [&](int i) {
+    const int quad = i / n_blocks;
+    T.blk = i - quad * n_blocks;
+    T.tl = quad * 4 + (lane & 3);
+    T.e = T.blk * 8 + (lane >> 2);
+    T.ok = T.tl < nt && T.e < n_elems;
+    T.t = t0 + min(T.tl, nt - 1);
+    if (EPI == CHAIN_QKV && T.ok) {
+      const int pr = (n0 >> 1) + T.e;  // weight rows 2 e and 2 e + 1 of the slab are a rotary pair (chain_qkv_row)
+      T.hh = pr >> (hl2 - 1);
+      T.j = pr & (half - 1);
+      const bf16* bias = G.bias + ((size_t)T.hh << hl2) + T.j;
+      T.bias = make_float2(__bfloat162float(bias[0]), __bfloat162float(bias[half]));
+      T.cs = make_float2(1.f, 0.f);
+      if (T.hh < G.Hq + G.Hkv) T.cs = __ldcg(reinterpret_cast<const float2*>(G.rope_cs + ((size_t)T.t << hl2) + 2 * T.j));
+      if (T.hh >= G.Hq) {  // the stream's slice of a contiguous cache, or its page
+        const int2 br = row_at(G.rm, T.t);
         const int pos = __ldcg(G.len + br.x) + br.y;
-        p.owner[q] = br.x;
-        p.slot[q] = pos;
+        T.owner = br.x;
+        T.slot = pos;
         if (pos < 0 || pos >= G.cap) {  // never write outside the stream's slice of the cache
           atomicOr(G.status, SSD_STATUS_KV_OVERFLOW);
-          p.slot[q] = -1;
+          T.slot = -1;
         } else if (G.page_table) {  // no page granted (pool exhausted): flagged by the page kernel
-          p.owner[q] = __ldcg(G.page_table + (size_t)br.x * G.max_pages + pos / TC_PAGE_TOKENS);
-          p.slot[q] = p.owner[q] < 0 ? -1 : pos % TC_PAGE_TOKENS;
+          T.owner = __ldcg(G.page_table + (size_t)br.x * G.max_pages + pos / TC_PAGE_TOKENS);
+          T.slot = T.owner < 0 ? -1 : pos % TC_PAGE_TOKENS;
         }
       }
     }
-  };
-  if (EPI == CHAIN_QKV && task0 < n_quads * (rows >> 1)) load_qkv(task0, qp);
-  // residual: RW lanes of a warp take RW weight rows of four token rows
-  const int RW = rows <= 8 ? 8 : rows <= 16 ? 16 : 32, rw = (rows + RW - 1) / RW, sublane = lane & (RW - 1);
-  struct ResTask {
-    int quad, rb;
-    float h[4], gain;
-  } rp;
-  rp.gain = 0.f;
-  auto load_res = [&](int i, ResTask& p) {  // i: task of this lane's group
-    p.quad = i / rw;
-    p.rb = i - p.quad * rw;
-    const int row = p.rb * RW + sublane, n = n0 + row;
-    p.gain = 0.f;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) p.h[q] = 0.f;
-    if (row < rows) {
-      p.gain = __bfloat162float(G.gain[n]);
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (p.quad * 4 + q < nt) p.h[q] = __ldcg(G.h + (size_t)(t0 + p.quad * 4 + q) * G.n_rows + n);
+    if (EPI == CHAIN_RESIDUAL) {
+      T.h = T.gain = 0.f;
+      if (T.ok) {
+        T.gain = __bfloat162float(G.gain[n0 + T.e]);
+        T.h = __ldcg(G.h + (size_t)T.t * G.n_rows + n0 + T.e);
+      }
     }
   };
-  const int res_step = CH_THREADS / RW, res0 = task0 / RW;
-  if (EPI == CHAIN_RESIDUAL && res0 < n_quads * rw) load_res(res0, rp);
+  if (EPI != CHAIN_SWIGLU && EPI != CHAIN_LOGITS && task0 < n_tasks) load_task(task0);
 
   // ---- the accumulator's columns to the owners of their token rows
   {
@@ -307,15 +307,15 @@ __global__ void __launch_bounds__(CH_THREADS) tc_chain_kernel(const __grid_const
           float* dst = mine + (size_t)o * P.rows_max * P.Tcp + tl;
 #pragma unroll
           for (int i = 0; i < 32; i += 4) {
-            if (c0 + i < M) {  // four token rows, all of one owner
-              *reinterpret_cast<float4*>(dst) =
-                  make_float4(__uint_as_float(v[i]) + __uint_as_float(w[i]), __uint_as_float(v[i + 1]) + __uint_as_float(w[i + 1]),
-                              __uint_as_float(v[i + 2]) + __uint_as_float(w[i + 2]), __uint_as_float(v[i + 3]) + __uint_as_float(w[i + 3]));
-              dst += 4;
-              if (C > 1 && (tl += 4) >= P.Tc) {
-                tl = 0;
-                dst += (size_t)P.rows_max * P.Tcp - P.Tc;
-              }
+            // four token rows, all of one owner (C = 1: room for whole ranges of 32)
+            if (C > 1 && c0 + i >= M) break;
+            *reinterpret_cast<float4*>(dst) =
+                make_float4(__uint_as_float(v[i]) + __uint_as_float(w[i]), __uint_as_float(v[i + 1]) + __uint_as_float(w[i + 1]),
+                            __uint_as_float(v[i + 2]) + __uint_as_float(w[i + 2]), __uint_as_float(v[i + 3]) + __uint_as_float(w[i + 3]));
+            dst += 4;
+            if (C > 1 && (tl += 4) >= P.Tc) {
+              tl = 0;
+              dst += (size_t)P.rows_max * P.Tcp - P.Tc;
             }
           }
         }
@@ -344,99 +344,37 @@ __global__ void __launch_bounds__(CH_THREADS) tc_chain_kernel(const __grid_const
     tmem_dealloc(tmem, P.tmem_cols);
   }
 
-  // ---- the C contributions of this CTA's token rows, in rank order, and what becomes of them.  A task is
-  // four token rows of one weight row (or of the two that belong together); the lanes of a warp are
-  // neighbouring weight rows, so that what they store is contiguous.
+  // ---- the C contributions of this CTA's token rows, in rank order, and what becomes of them
   const int src = P.rows_max * P.Tcp;  // floats from one CTA's contributions to the next one's
-  auto sum4 = [&](int row, int quad) {
-    const float* r = red + (size_t)row * P.Tcp + quad * 4;
-    float4 a = *reinterpret_cast<const float4*>(r);
+  auto sum = [&](int row, int tl) {
+    const float* r = red + row * P.Tcp + tl;
+    float a = r[0];
     if (C == 8) {  // all loads in flight
-      float4 b[7];
+      float b[7];
 #pragma unroll
-      for (int s = 0; s < 7; ++s) b[s] = *reinterpret_cast<const float4*>(r + (s + 1) * src);
+      for (int s = 0; s < 7; ++s) b[s] = r[(s + 1) * src];
 #pragma unroll
-      for (int s = 0; s < 7; ++s) {
-        a.x += b[s].x; a.y += b[s].y; a.z += b[s].z; a.w += b[s].w;
-      }
+      for (int s = 0; s < 7; ++s) a += b[s];
     }
     return a;
   };
-  if (n_quads > 0 && !*abort) {
-    if (EPI == CHAIN_QKV) {
-      for (int i = task0; i < n_quads * (rows >> 1); i += CH_THREADS) {
-        if (i != task0) load_qkv(i, qp);
-        const int quad = qp.quad, e = qp.e, hh = qp.hh, j = qp.j;
-        const float4 xs = sum4(2 * e, quad), ys = sum4(2 * e + 1, quad);
-        const float x4[4] = {xs.x, xs.y, xs.z, xs.w}, y4[4] = {ys.x, ys.y, ys.z, ys.w};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int tl = quad * 4 + q, t = t0 + tl;
-          if (tl >= nt) break;
-          const float inv = S.inv_rms[tl];
-          const float x = fmaf(x4[q], inv, qp.bx), y = fmaf(y4[q], inv, qp.by);
-          const float u = x * qp.cs[q].x - y * qp.cs[q].y, v = y * qp.cs[q].x + x * qp.cs[q].y;  // values: (1, 0), unchanged
-          if (hh < G.Hq) {
-            float* dst = G.qrot + (((size_t)t * G.Hq + hh) << hl2) + j;
-            dst[0] = u * G.qscale;
-            dst[half] = v * G.qscale;
-          } else if (qp.slot[q] >= 0) {
-            const int which = hh >= G.Hq + G.Hkv, g = hh - G.Hq - which * G.Hkv;
-            bf16* dst = G.kv_layer + (((((size_t)qp.owner[q] * 2 + which) * G.Hkv + g) * rows_per + qp.slot[q]) << hl2) + j;
-            dst[0] = __float2bfloat16_rn(u);
-            dst[half] = __float2bfloat16_rn(v);
-          }
-        }
-      }
-    } else if (EPI == CHAIN_RESIDUAL) {
-      // the rows' sums of squares by shuffles; all lanes of a warp make the same number of passes
-      float* sq = &S.inv_rms[0];  // [token][rw]: not in use by this epilogue
-      const int n_tasks = n_quads * rw, passes = (n_tasks + res_step - 1) / res_step;
-      for (int pass = 0; pass < passes; ++pass) {
-        const int i = res0 + pass * res_step;
-        const bool have = i < n_tasks;
-        if (pass > 0 && have) load_res(i, rp);
-        if (!have) rp.quad = rp.rb = 0;
-        const int quad = rp.quad, row = rp.rb * RW + sublane, n = n0 + row, valid = min(4, nt - quad * 4);
-        const bool ok = have && row < rows;
-        float hv[4] = {0.f, 0.f, 0.f, 0.f}, x[4];
-        float* hp = G.h + (size_t)(t0 + quad * 4) * G.n_rows + n;
-        if (ok) {
-          const float4 a = sum4(row, quad);
-          hv[0] = rp.h[0] + a.x; hv[1] = rp.h[1] + a.y; hv[2] = rp.h[2] + a.z; hv[3] = rp.h[3] + a.w;
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (q < valid) hp[(size_t)q * G.n_rows] = hv[q];
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) x[q] = hv[q] * rp.gain;
-        store_pair4(G.lay_out, G.act_out, t0 + quad * 4, n & ~1, lane, x, ok ? valid : 0);
-        float ss[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) ss[q] = q < valid ? hv[q] * hv[q] : 0.f;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          if (o < RW) {  // uniform
-#pragma unroll
-            for (int q = 0; q < 4; ++q) ss[q] += __shfl_xor_sync(0xffffffffu, ss[q], o);
-          }
-        }
-        if (sublane == 0 && have) {
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (q < valid) sq[(quad * 4 + q) * rw + rp.rb] = ss[q];
-        }
-      }
-      __syncthreads();  // (every thread of the CTA is here)
-      if (tid < nt) {
-        float v = 0.f;
-        for (int e = 0; e < rw; ++e) v += sq[tid * rw + e];
-        G.ssq_out[(size_t)cl * P.Mpad + t0 + tid] = v;
-      }
-    } else if (EPI == CHAIN_SWIGLU) {
-      const int per = rows >> 1, n_tasks = n_quads * per;  // rows interleaved: gate, up; per is a multiple of 4
-      for (int i0 = warp * 32; i0 < n_tasks; i0 += CH_THREADS) {
-        const int i = min(i0 + lane, n_tasks - 1), quad = i / per, e = i - quad * per, k = (n0 >> 1) + e;
+  auto sum4 = [&](int row, int quad) {  // of four token rows
+    const float* r = red + row * P.Tcp + quad * 4;
+    float4 a = *reinterpret_cast<const float4*>(r);
+    for (int s = 1; s < C; ++s) {
+      const float4 b = *reinterpret_cast<const float4*>(r + s * src);
+      a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
+    }
+    return a;
+  };
+  if (!*abort) {
+    float* sq = &S.inv_rms[0];  // residual: [token][block] sums of squares (1/rms is not in use by that epilogue)
+    if (EPI == CHAIN_SWIGLU) {
+      // every CTA has hundreds of elements here: four token rows per thread (one per thread: 10.5 instead of
+      // 8.9 us at 96 rows); lanes are neighbouring columns
+      const int per = rows >> 1, n_all = n_quads * per;  // rows interleaved: gate, up; per is a multiple of 4
+      for (int i0 = warp * 32; i0 < n_all; i0 += CH_THREADS) {
+        const int i = min(i0 + lane, n_all - 1), quad = i / per, e = i - quad * per, k = (n0 >> 1) + e;
         const float4 g = sum4(2 * e, quad), u = sum4(2 * e + 1, quad);
         const float4 inv = *reinterpret_cast<const float4*>(&S.inv_rms[quad * 4]);
         const float g4[4] = {g.x * inv.x, g.y * inv.y, g.z * inv.z, g.w * inv.w};
@@ -444,9 +382,9 @@ __global__ void __launch_bounds__(CH_THREADS) tc_chain_kernel(const __grid_const
         float x[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) x[q] = __fdividef(g4[q], 1.f + __expf(-g4[q])) * u4[q];
-        store_pair4(G.lay_out, G.act_out, t0 + quad * 4, k & ~1, lane, x, i0 + lane < n_tasks ? min(4, nt - quad * 4) : 0);
+        store_pair4(G.lay_out, G.act_out, t0 + quad * 4, k & ~1, lane, x, i0 + lane < n_all ? min(4, nt - quad * 4) : 0);
       }
-    } else {
+    } else if (EPI == CHAIN_LOGITS) {
       for (int i = tid; i < n_quads * rows; i += CH_THREADS) {
         const int quad = i / rows, e = i - quad * rows;
         const float4 a = sum4(e, quad);
@@ -456,6 +394,50 @@ __global__ void __launch_bounds__(CH_THREADS) tc_chain_kernel(const __grid_const
           const int tl = quad * 4 + q;
           if (tl < nt && n0 + e < G.n_rows) G.out[(size_t)(t0 + tl) * G.n_rows + n0 + e] = a4[q] * S.inv_rms[tl];
         }
+      }
+    } else {
+#pragma unroll 1
+    for (int i = task0; i < n_tasks; i += CH_THREADS / 32) {
+      if (i != task0) load_task(i);
+      if (EPI == CHAIN_QKV) {
+        if (T.ok) {
+          const float inv = S.inv_rms[T.tl];
+          const float x = fmaf(sum(2 * T.e, T.tl), inv, T.bias.x), y = fmaf(sum(2 * T.e + 1, T.tl), inv, T.bias.y);
+          const float u = x * T.cs.x - y * T.cs.y, v = y * T.cs.x + x * T.cs.y;  // values: (1, 0), unchanged
+          if (T.hh < G.Hq) {
+            float* dst = G.qrot + (((size_t)T.t * G.Hq + T.hh) << hl2) + T.j;
+            dst[0] = u * G.qscale;
+            dst[half] = v * G.qscale;
+          } else if (T.slot >= 0) {
+            const int which = T.hh >= G.Hq + G.Hkv, g = T.hh - G.Hq - which * G.Hkv;
+            const size_t rows_per = G.page_table ? (size_t)TC_PAGE_TOKENS : (size_t)G.cap;
+            bf16* dst = G.kv_layer + (((((size_t)T.owner * 2 + which) * G.Hkv + g) * rows_per + T.slot) << hl2) + T.j;
+            dst[0] = __float2bfloat16_rn(u);
+            dst[half] = __float2bfloat16_rn(v);
+          }
+        }
+      } else if (EPI == CHAIN_RESIDUAL) {
+        const int n = n0 + T.e;
+        float x = 0.f;
+        if (T.ok) {
+          x = T.h + sum(T.e, T.tl);
+          G.h[(size_t)T.t * G.n_rows + n] = x;
+        }
+        store_shared(G.lay_out.row(G.act_out, T.t), G.lay_out, n, x * T.gain, T.ok);
+        float ss = x * x;
+        ss += __shfl_xor_sync(0xffffffffu, ss, 4);
+        ss += __shfl_xor_sync(0xffffffffu, ss, 8);
+        ss += __shfl_xor_sync(0xffffffffu, ss, 16);
+        if (lane < 4 && T.ok) sq[T.tl * n_blocks + T.blk] = ss;
+      }
+    }
+    }
+    if (EPI == CHAIN_RESIDUAL) {
+      __syncthreads();  // (every thread of the CTA is here)
+      if (tid < nt) {
+        float v = 0.f;
+        for (int e = 0; e < n_blocks; ++e) v += sq[tid * n_blocks + e];
+        G.ssq_out[(size_t)cl * P.Mpad + t0 + tid] = v;
       }
     }
   }
@@ -597,7 +579,8 @@ cudaError_t launch_tc_chain(const ChainGemm& g, int epi, int K, bool whole, int 
   p.Mc = cs.tsplit > 1 ? chain_chunk_rows(g.M, K, whole) : p.Mpad;
   const int Mcta = cs.tsplit > 1 ? p.Mc : g.M;
   p.Tc = ((Mcta + cs.cluster - 1) / cs.cluster + 3) / 4 * 4;  // quads of token rows have one owner
-  p.Tcp = p.Tc % 8 == 4 ? p.Tc : p.Tc + 4;                   // 16-byte stores of 8 lanes to 32 banks
+  p.Tcp = cs.cluster > 1 ? p.Tc : (p.Tc + 31) / 32 * 32;
+  if (p.Tcp % 8 == 0) p.Tcp += 4;                            // 16-byte stores of 8 lanes to 32 banks
   p.ng_max = (p.n_groups + cs.clusters - 1) / cs.clusters;
   p.rows_max = p.ng_max * 8;
   const size_t red = (size_t)cs.cluster * p.Tcp * p.rows_max * 4 * (cs.cluster > 1 ? 2 : 1);  // gathered, and pushed
