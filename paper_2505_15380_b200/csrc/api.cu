@@ -149,8 +149,8 @@ size_t blob_elems(const ssd_model_config& c) {
 }
 
 struct WsPlan {
-  size_t len, pending, status, counters, row_ids, accept_flags;
-  size_t h, qkv, qrot, rope_cs, part, logits, row_stats, xn, attn_out, act;
+  size_t len, pending, status, counters, row_ids, row_words;
+  size_t h, qkv, qrot, rope_cs, part, logits, xn, attn_out, act;
   size_t st_tokens, st_k, st_y, st_probs, st_uni;
   size_t hfix, flags, epoch_base, xa, xb, xd, xq, ssq_a, ssq_b;
   size_t ch_ssq_a, ch_ssq_b, tc_rowmap, tc_tiles, tc_xa, tc_xattn, tc_xact, tc_part;
@@ -187,14 +187,13 @@ WsPlan plan_ws(const ssd_model_config& c, int B, int max_gamma, int cap, int n_p
   p.status = take(4);
   p.counters = take(B * 4);
   p.row_ids = take(MX * 4);
-  p.accept_flags = take(M * 4);
+  p.row_words = take(M * 4);
   p.h = take(MX * d * 4);
   p.qkv = take(M * (qd + 2 * kvd) * 4);
   p.qrot = take(MX * qd * 4);
   p.rope_cs = take(MX * c.head_dim * 4);
   p.part = take(MP * c.n_q_heads * (size_t)p.nsplit_max * (c.head_dim + 2) * 4);
   p.logits = take(M * V * 4);
-  p.row_stats = take(M * 8 * 4);  // eight statistics words per row (sampler.cu)
   p.xn = take(M * d * 4);
   p.attn_out = take(M * qd * 4);
   p.act = take(M * F * 4);
@@ -280,9 +279,18 @@ bool same_shape(const ssd_model_config& a, const ssd_model_config& b) {
 
 // One decoder forward over the rows described by rm (ids already in s->row_ids).  Appends the
 // rows' K/V at len + r; when logits_out is non-null also runs the final norm and the LM head.
-// The persistent kernel covers forwards of at most FAST_MAX_T rows over a bf16 model.
-bool use_fast(const ssd_model* m, const ssd_streams* s, RowMap rm) {
-  return m->fast.enabled && s->path == 0 && !s->paged && !rm.rows && rm.nb * rm.R <= (rm.nb > 1 ? 8 : FAST_MAX_T);
+// The persistent kernel covers forwards of at most FAST_MAX_T rows over a bf16 model.  Of 9 to 16 rows
+// over several streams it takes none (its CTAs repeat every stream's attention: 12 rows of 3 streams
+// 1.07 ms against 0.86 as a chain), unless the rows are for a nucleus over the whole vocabulary: that cut
+// falls among ids about 3e-4 apart, so the 1e-4 by which another order of summation moves a logit
+// changes a few per cent of the draws, and such streams keep the sums they have always had.
+bool use_fast(const ssd_model* m, const ssd_streams* s, RowMap rm, bool whole_nucleus = false) {
+  return m->fast.enabled && s->path == 0 && !s->paged && !rm.rows &&
+         rm.nb * rm.R <= (rm.nb > 1 && !whole_nucleus ? 8 : FAST_MAX_T);
+}
+// A nucleus that no top-k bounds.
+bool whole_nucleus(const ssd_verify_params* p, int V) {
+  return p->top_p > 0.f && p->top_p < 1.f && (p->top_k <= 0 || p->top_k >= V);
 }
 
 int forward_fast(const ssd_model* m, ssd_streams* s, RowMap rm, const int32_t* row_ids,
@@ -1009,14 +1017,13 @@ int streams_create_impl(const ssd_model* m, int32_t batch, int32_t capacity_toke
   s->status = (int32_t*)(W + p.status);
   s->counters = (int32_t*)(W + p.counters);
   s->row_ids = (int32_t*)(W + p.row_ids);
-  s->accept_flags = (int32_t*)(W + p.accept_flags);
+  s->row_words = (int32_t*)(W + p.row_words);
   s->h = (float*)(W + p.h);
   s->qkv = (float*)(W + p.qkv);
   s->qrot = (float*)(W + p.qrot);
   s->rope_cs = (float*)(W + p.rope_cs);
   s->part = (float*)(W + p.part);
   s->logits = (float*)(W + p.logits);
-  s->row_stats = (float*)(W + p.row_stats);
   s->xn = (float*)(W + p.xn);
   s->attn_out = (float*)(W + p.attn_out);
   s->act = (float*)(W + p.act);
@@ -1297,7 +1304,7 @@ int verify_impl(ssd_model* target, ssd_streams* s, const int32_t* dev_draft_toke
   float* logits = dev_logits_or_null ? dev_logits_or_null : s->logits;
   const RowMap rm{0, s->B, gamma + 1};
   int rc;
-  if (use_fast(target, s, rm)) {
+  if (use_fast(target, s, rm, whole_nucleus(params, target->cfg.vocab_out))) {
     rc = forward_fast(target, s, rm, nullptr, dev_draft_tokens, logits, st);
   } else if (use_chain(target, s, rm)) {
     rc = forward_chain(target, s, rm, dev_draft_tokens, logits, st);
@@ -1315,7 +1322,7 @@ int verify_impl(ssd_model* target, ssd_streams* s, const int32_t* dev_draft_toke
   SSD_CUDA(launch_verify_sampler(logits, target->cfg.vocab_out, dev_draft_tokens, dev_draft_probs,
                                  dev_uniforms, s->B, gamma, 1.0f / params->temperature,
                                  params->top_k, params->top_p, params->beta, params->ras_window, params->ras_tau,
-                                 params->dev_recent_tokens, s->row_stats, s->accept_flags,
+                                 params->dev_recent_tokens, s->row_words,
                                  s->counters, dev_accepted_len, dev_next_token, s->status, st));
   return SSD_OK;
 }

@@ -139,8 +139,8 @@ struct ssd_streams {
   char* ws;
   size_t ws_bytes;
   // regions of the workspace
-  int32_t *len, *pending, *status, *counters, *row_ids, *accept_flags;
-  float *h, *qkv, *qrot, *rope_cs, *part, *logits, *row_stats, *xn, *attn_out, *act;
+  int32_t *len, *pending, *status, *counters, *row_ids, *row_words;
+  float *h, *qkv, *qrot, *rope_cs, *part, *logits, *xn, *attn_out, *act;
   // staging for the host-buffer entry point
   int32_t *st_tokens, *st_k, *st_y;
   float *st_probs, *st_uni;

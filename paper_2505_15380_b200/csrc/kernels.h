@@ -54,7 +54,7 @@ cudaError_t launch_verify_sampler(const float* logits, int V, const int32_t* dra
                                   const float* draft_probs, const float* uniforms, int B,
                                   int gamma, float inv_temperature, int top_k, float top_p, float beta,
                                   int ras_window, float ras_tau, const int32_t* recent_tokens,
-                                  float* row_stats, int32_t* accept_flags, int32_t* counters,
+                                  int32_t* row_words, int32_t* counters,
                                   int32_t* accepted_len, int32_t* next_token, int32_t* status,
                                   cudaStream_t st);
 // out_token[b * tok_stride] and out_prob_row[b * prob_stride + t]: the strides let a loop write

@@ -1,8 +1,12 @@
 // Fused logits -> sampling transform -> acceptance test -> residual resample / bonus draw
 // (Algorithm 1's inner loop, Eq. 5 and Eq. 6), plus the KV commit.  Probability rows q_i never
-// reach global memory: each (stream, row) CTA keeps its row in shared memory and leaves only four
-// words of statistics; the CTA that finishes last for a stream reduces the accept flags to the
-// accepted length k, rebuilds row k on chip and draws the new token.
+// reach global memory: each (stream, row) CTA keeps its row in shared memory, tests its draft token
+// and draws the token that would follow if this were the first rejected row; it leaves one word.  The CTA
+// that finishes last for a stream picks the accepted length k and row k's token.
+//
+// What bounds it: the chain of trips to memory and block barriers of ONE row (6564 logits are seven per
+// thread), not bytes.  So every row draws ahead of the decision (rereading row k afterwards cost three
+// more trips to L2), block reductions take two warp steps, and the cuts below one histogram pass.
 //
 // p = DRAFT distribution, q = TARGET distribution, as in the paper.
 #include <math_constants.h>
@@ -28,28 +32,20 @@ __device__ __forceinline__ uint32_t order_key(float f) {
   uint32_t u = __float_as_uint(f);
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
+__device__ __forceinline__ float key_value(uint32_t k) { return __uint_as_float(k & 0x80000000u ? k & 0x7fffffffu : ~k); }
 __device__ __forceinline__ bool is_kept(float z, int t, const RowStats& s) {
   uint32_t k = order_key(z);
   return k > s.thr_key || (k == s.thr_key && t <= s.tie_id_max);
 }
 
-__device__ __forceinline__ float block_max(float v, float* red) {
-  v = warp_max(v);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+// Sums of two values over the block, in every thread: lanes, then warps (fixed order).
+__device__ __forceinline__ double2 block_sum_d(double a, double b, bool two, double2* red) {
+  a = warp_sum_d(a);
+  if (two) b = warp_sum_d(b);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_double2(a, b);
   __syncthreads();
-  float r = red[0];
-  for (int i = 1; i < SAMP_THREADS / 32; ++i) r = fmaxf(r, red[i]);
-  __syncthreads();
-  return r;
-}
-__device__ __forceinline__ double block_sum_d(double v, double* red) {
-  v = warp_sum_d(v);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double r = 0.0;
-  for (int i = 0; i < SAMP_THREADS / 32; ++i) r += red[i];
-  __syncthreads();
-  return r;
+  const double2 v = red[threadIdx.x & 31];
+  return make_double2(warp_sum_d(v.x), two ? warp_sum_d(v.y) : 0.0);
 }
 
 __device__ __forceinline__ unsigned long long block_sum_u64(unsigned long long v, unsigned long long* red) {
@@ -70,7 +66,6 @@ __device__ __forceinline__ unsigned long long mass_fx(float x) { return __float2
 // win * tau times is thrown away and redrawn from the full softmax.  As one distribution:
 //   q(x) = q_nuc(x) [x not repeated] + R q_full(x),  R = mass of q_nuc on the repeated ids.
 constexpr int RAS_MAX_WIN = 32;
-constexpr int RS_STRIDE = 8;  // floats of row statistics per row: the four of RowStats, sum_full, R
 struct Ras {
   int win;               // 0: off
   float thresh;          // win * tau
@@ -81,28 +76,231 @@ struct RasRow {
   float R;
 };
 
+constexpr int SEL_BINS = 512;  // bins of a row's range of values, for the cuts
+constexpr int SEL_CAND = 512;  // most ids of the bin in which a cut falls that are ranked one by one
+
 struct SampSmem {
   int rep_ids[RAS_MAX_WIN];  // repeated ids of this row's window (-1: none)
+  uint32_t cnt[SEL_BINS];                 // ids per bin
+  uint32_t mass_lo[SEL_BINS], mass_hi[SEL_BINS];  // their mass, low 16 bits and the rest (32-bit atomics, no carries)
+  union {  // the cuts' candidates; later the draw's running sums
+    struct {
+      unsigned long long cand_mass[SEL_CAND];
+      uint32_t cand_key[SEL_CAND];
+      int cand_id[SEL_CAND];
+    };
+    double scan[SAMP_THREADS];
+  };
   unsigned long long hist_fx[256];
   unsigned long long red_u[SAMP_THREADS / 32];
-  unsigned long long mass_above;
+  unsigned long long mass_above, target;
+  double2 red_d2[SAMP_THREADS / 32];
   double red_d[SAMP_THREADS / 32];
-  double scan[SAMP_THREADS];
-  float red_f[SAMP_THREADS / 32];
+  uint32_t red_max[SAMP_THREADS / 32], red_min[SAMP_THREADS / 32];
   int hist[256];
-  uint32_t prefix;
-  int k_rem, eq_count, tie_id, bad, last, k_acc, y;
+  uint32_t prefix, cut;
+  int k_rem, eq_count, tie_id, cut_id, sel_bin, n_cand, y;
 };
 
-// Row statistics of the sampling transform: z/T is already in `z` (shared).  Block-collective.
-__device__ RowStats compute_row_stats(const float* z, int V, int top_k, float top_p, SampSmem& sm) {
-  RowStats st;
-  float mx = -CUDART_INF_F;
-  for (int t = threadIdx.x; t < V; t += SAMP_THREADS) mx = fmaxf(mx, z[t]);
-  st.zmax = block_max(mx, sm.red_f);
-  st.thr_key = 0u;
-  st.tie_id_max = V;
-  if (top_k > 0 && top_k < V) {
+// A row's values by size in bins of equal width, bin 0 the largest: monotone, so a cut falls in one bin.
+struct BinMap {
+  float zmax, scale;
+  bool ok;  // a finite range (else the cuts use the bits of the values)
+  __device__ __forceinline__ int operator()(float z) const {
+    return min((int)__fmul_rn(__fsub_rn(zmax, z), scale), SEL_BINS - 1);
+  }
+};
+
+// Before the row arrives: nothing is counted yet.  The load's barrier publishes it.
+__device__ __forceinline__ void clear_bins(SampSmem& sm) {
+  for (int i = threadIdx.x; i < SEL_BINS; i += SAMP_THREADS) sm.cnt[i] = sm.mass_lo[i] = sm.mass_hi[i] = 0u;
+}
+
+// A row of logits to z / T in shared memory; its range.  Block-collective.
+__device__ __forceinline__ BinMap load_row(const float* __restrict__ lrow, int V, float inv_t, float* z, SampSmem& sm,
+                                           int32_t* status) {
+  float mx = -CUDART_INF_F, mn = CUDART_INF_F;
+  int bad = 0;
+#pragma unroll 8
+  for (int t = threadIdx.x; t < V; t += SAMP_THREADS) {
+    const float v = lrow[t];
+    if (!isfinite(v)) bad = 1;
+    const float x = v * inv_t;
+    z[t] = x;
+    mx = fmaxf(mx, x);
+    mn = fminf(mn, x);
+  }
+  const uint32_t kmx = __reduce_max_sync(0xffffffffu, order_key(mx)), kmn = __reduce_min_sync(0xffffffffu, order_key(mn));
+  if ((threadIdx.x & 31) == 0) {
+    sm.red_max[threadIdx.x >> 5] = kmx;
+    sm.red_min[threadIdx.x >> 5] = kmn;
+  }
+  bad = __syncthreads_or(bad);
+  if (bad && threadIdx.x == 0) atomicOr(status, SSD_STATUS_NONFINITE);
+  BinMap m;
+  m.zmax = key_value(__reduce_max_sync(0xffffffffu, sm.red_max[threadIdx.x & 31]));
+  const float range = m.zmax - key_value(__reduce_min_sync(0xffffffffu, sm.red_min[threadIdx.x & 31]));
+  m.ok = !bad && range > 1e-20f && range < 1e30f;
+  m.scale = (float)SEL_BINS / range;
+  return m;
+}
+
+// Both cuts: one pass counts ids (or adds up masses) per bin, one warp finds the bin in which the cut
+// falls, a second pass lists that bin's ids, and each of those finds its own place among them.  A radix select
+// over the bits of the values took four passes and, since the top eight bits of a row take a handful of values,
+// serialised its shared-memory atomics.  Rows that do not spread over the bins (more than SEL_CAND ids
+// in that one, e.g. many equal values) still take it.
+
+// The top_k-th largest id (lower id first among equals).  False: not found this way.
+__device__ bool cut_by_count(const float* z, int V, int top_k, const BinMap& map, SampSmem& sm, RowStats& st) {
+  const int tid = threadIdx.x;
+  for (int t = tid; t < V; t += SAMP_THREADS) atomicAdd(&sm.cnt[map(z[t])], 1u);
+  __syncthreads();
+  if (tid < 32) {
+    constexpr int PER = SEL_BINS / 32;
+    uint32_t h[PER], tot = 0;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) tot += h[i] = sm.cnt[PER * tid + i];
+    uint32_t run = tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, run, o);
+      if (tid >= o) run += v;
+    }
+    run -= tot;
+    if (run < (uint32_t)top_k && run + tot >= (uint32_t)top_k) {
+      bool found = false;
+#pragma unroll
+      for (int i = 0; i < PER; ++i) {
+        if (!found && run + h[i] >= (uint32_t)top_k) {
+          found = true;
+          sm.sel_bin = PER * tid + i;
+          sm.k_rem = top_k - (int)run;
+        }
+        run += h[i];
+      }
+    }
+    if (tid == 0) sm.n_cand = 0;
+  }
+  __syncthreads();
+  const int sel = sm.sel_bin;
+  for (int t = tid; t < V; t += SAMP_THREADS) {
+    const float x = z[t];
+    if (map(x) == sel) {
+      const int i = atomicAdd(&sm.n_cand, 1);
+      if (i < SEL_CAND) {
+        sm.cand_key[i] = order_key(x);
+        sm.cand_id[i] = t;
+      }
+    }
+  }
+  __syncthreads();
+  const int n = sm.n_cand;
+  if (n > SEL_CAND) return false;
+  if (tid < n) {
+    const uint32_t key = sm.cand_key[tid];
+    const int id = sm.cand_id[tid];
+    int before = 0;
+    for (int i = 0; i < n; ++i) before += sm.cand_key[i] > key || (sm.cand_key[i] == key && sm.cand_id[i] < id);
+    if (before == sm.k_rem - 1) {
+      sm.cut = key;
+      sm.cut_id = id;
+    }
+  }
+  __syncthreads();
+  st.thr_key = sm.cut;
+  st.tie_id_max = sm.cut_id;
+  return true;
+}
+
+// The id at which the running mass of the kept ids first reaches top_p of their mass.
+__device__ bool cut_by_mass(const float* z, int V, float top_p, const BinMap& map, SampSmem& sm, RowStats& st) {
+  const int tid = threadIdx.x;
+  for (int t = tid; t < V; t += SAMP_THREADS) {
+    const float x = z[t];
+    if (is_kept(x, t, st)) {
+      const unsigned long long m = mass_fx(x - st.zmax);
+      const int b = map(x);
+      if (m) {  // (V is below 2^16: neither word overflows)
+        atomicAdd(&sm.mass_lo[b], (uint32_t)m & 0xffffu);
+        atomicAdd(&sm.mass_hi[b], (uint32_t)(m >> 16));
+      }
+    }
+  }
+  __syncthreads();
+  if (tid < 32) {
+    constexpr int PER = SEL_BINS / 32;
+    auto mass = [&](int i) { return (unsigned long long)sm.mass_lo[PER * tid + i] + ((unsigned long long)sm.mass_hi[PER * tid + i] << 16); };
+    unsigned long long tot = 0;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) tot += mass(i);
+    unsigned long long run = tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long v = __shfl_up_sync(0xffffffffu, run, o);
+      if (tid >= o) run += v;
+    }
+    const unsigned long long total = __shfl_sync(0xffffffffu, run, 31);
+    run -= tot;
+    const double td = (double)top_p * (double)total;
+    unsigned long long target = (unsigned long long)td;
+    if ((double)target < td) ++target;  // an id stays iff (mass before it) < target
+    if (target < 1) target = 1;
+    if (run < target && run + tot >= target) {
+      bool found = false;
+#pragma unroll
+      for (int i = 0; i < PER; ++i) {
+        const unsigned long long h = mass(i);
+        if (!found && run + h >= target) {
+          found = true;
+          sm.sel_bin = PER * tid + i;
+          sm.mass_above = run;
+        }
+        run += h;
+      }
+    }
+    if (tid == 0) {
+      sm.target = target;
+      sm.n_cand = 0;
+    }
+  }
+  __syncthreads();
+  const int sel = sm.sel_bin;
+  for (int t = tid; t < V; t += SAMP_THREADS) {
+    const float x = z[t];
+    if (map(x) == sel && is_kept(x, t, st)) {
+      const int i = atomicAdd(&sm.n_cand, 1);
+      if (i < SEL_CAND) {
+        sm.cand_key[i] = order_key(x);
+        sm.cand_id[i] = t;
+        sm.cand_mass[i] = mass_fx(x - st.zmax);
+      }
+    }
+  }
+  __syncthreads();
+  const int n = sm.n_cand;
+  if (n > SEL_CAND) return false;
+  if (tid < n) {
+    const uint32_t key = sm.cand_key[tid];
+    const int id = sm.cand_id[tid];
+    unsigned long long before = sm.mass_above;
+    for (int i = 0; i < n; ++i)
+      if (sm.cand_key[i] > key || (sm.cand_key[i] == key && sm.cand_id[i] < id)) before += sm.cand_mass[i];
+    if (before < sm.target && before + sm.cand_mass[tid] >= sm.target) {
+      sm.cut = key;
+      sm.cut_id = id;
+    }
+  }
+  __syncthreads();
+  st.thr_key = sm.cut;
+  st.tie_id_max = sm.cut_id;
+  return true;
+}
+
+// The same cuts by a radix select over the bits of the values.
+__device__ __noinline__ void radix_cut_by_count(const float* z, int V, int top_k, SampSmem& sm, RowStats& st) {
+  {
+    __syncthreads();
     // radix select (4 passes of 8 bits, most significant first) of the top_k-th largest key
     if (threadIdx.x == 0) { sm.prefix = 0u; sm.k_rem = top_k; }
     for (int pass = 0; pass < 4; ++pass) {
@@ -163,7 +361,10 @@ __device__ RowStats compute_row_stats(const float* z, int V, int top_k, float to
     }
     __syncthreads();
   }
-  if (top_p > 0.f && top_p < 1.f) {
+}
+__device__ __noinline__ void radix_cut_by_mass(const float* z, int V, float top_p, SampSmem& sm, RowStats& st) {
+  {
+    __syncthreads();
     // Nucleus: walking the kept ids from the most to the least probable (lower id first among
     // equals), an id stays while the mass before it is below top_p of the kept mass.  The id at
     // which the running mass first reaches that target is found by a radix select over the
@@ -254,10 +455,37 @@ __device__ RowStats compute_row_stats(const float* z, int V, int top_k, float to
     st.tie_id_max = sm.tie_id;
     __syncthreads();
   }
-  double s = 0.0;
-  for (int t = threadIdx.x; t < V; t += SAMP_THREADS)
-    if (is_kept(z[t], t, st)) s += (double)expf(z[t] - st.zmax);
-  st.sum = (float)block_sum_d(s, sm.red_d);
+}
+
+// exp(z - zmax) of an id, negative where the id is cut off (zero there unless `full`).
+__device__ __forceinline__ float signed_exp(float z, int t, const RowStats& st, bool full) {
+  const bool kept = is_kept(z, t, st);
+  if (!kept && !full) return 0.f;
+  const float e = expf(z - st.zmax);
+  return kept ? e : -e;
+}
+
+// Row statistics of the sampling transform of a loaded row, and the sum over all ids where `full` asks for it;
+// z becomes signed_exp.  Block-collective.
+__device__ __forceinline__ RowStats compute_row_stats(float* z, int V, int top_k, float top_p, const BinMap& map,
+                                                      bool full, float* sum_full, SampSmem& sm) {
+  RowStats st;
+  st.zmax = map.zmax;
+  st.thr_key = 0u;
+  st.tie_id_max = V;
+  if (top_k > 0 && top_k < V && !(map.ok && cut_by_count(z, V, top_k, map, sm, st))) radix_cut_by_count(z, V, top_k, sm, st);
+  if (top_p > 0.f && top_p < 1.f && !(map.ok && cut_by_mass(z, V, top_p, map, sm, st))) radix_cut_by_mass(z, V, top_p, sm, st);
+  double s = 0.0, f = 0.0;
+#pragma unroll 4
+  for (int t = threadIdx.x; t < V; t += SAMP_THREADS) {
+    const float v = signed_exp(z[t], t, st, full);
+    z[t] = v;
+    if (v > 0.f) s += (double)v;
+    if (full) f += (double)fabsf(v);
+  }
+  const double2 sums = block_sum_d(s, f, full, sm.red_d2);
+  st.sum = (float)sums.x;
+  *sum_full = (float)sums.y;
   return st;
 }
 
@@ -326,60 +554,49 @@ __device__ int block_inverse_cdf(const float* w, int V, float u, SampSmem& sm, d
 }
 
 // The repeated ids of row r's window: the last `win` tokens of recent[b] ++ x_1..x_r (row r's
-// own token x_{r+1} is not part of it).  Block-collective; leaves them in sm.rep_ids.
-__device__ void ras_window(const Ras& ras, const int32_t* __restrict__ draft_tokens, int gamma, int b, int r, int V,
-                           SampSmem& sm) {
-  const int j = threadIdx.x;
-  if (j < RAS_MAX_WIN) {
-    int rep = -1;
-    if (j < ras.win) {
-      auto at = [&](int i) {  // i-th token of the window
-        const int c = r + i;
-        return c < ras.win ? ras.recent[(size_t)b * ras.win + c] : draft_tokens[b * gamma + c - ras.win];
-      };
-      const int t = at(j);
-      if (t >= 0 && t < V) {
-        int cnt = 0;
-        bool first = true;
-        for (int i = 0; i < ras.win; ++i) {
-          const bool same = at(i) == t;
-          cnt += same;
-          if (same && i < j) first = false;
-        }
-        if (first && (float)cnt >= ras.thresh) rep = t;
-      }
-    }
-    sm.rep_ids[j] = rep;
+// own token x_{r+1} is not part of it).  One warp; leaves them in sm.rep_ids.
+__device__ __forceinline__ void ras_window(const Ras& ras, const int32_t* __restrict__ draft_tokens, int gamma, int b, int r,
+                                           int V, SampSmem& sm) {
+  const int j = threadIdx.x & 31, c = r + j;  // lane j: j-th token of the window
+  int t = -1;
+  if (j < ras.win) t = c < ras.win ? ras.recent[(size_t)b * ras.win + c] : draft_tokens[b * gamma + c - ras.win];
+  int cnt = 0;
+  bool first = true;
+  for (int i = 0; i < ras.win; ++i) {
+    const bool same = __shfl_sync(0xffffffffu, t, i) == t;
+    cnt += same;
+    if (same && i < j) first = false;
   }
-  __syncthreads();
+  sm.rep_ids[j] = j < ras.win && t >= 0 && t < V && first && (float)cnt >= ras.thresh ? t : -1;
 }
 __device__ __forceinline__ bool ras_is_rep(const SampSmem& sm, int win, int t) {
   bool rep = false;
   for (int j = 0; j < win; ++j) rep |= sm.rep_ids[j] == t;
   return rep;
 }
-// sum_full and R of a row whose nucleus statistics are `st`.  Block-collective.
-__device__ RasRow ras_row(const float* z, int V, const RowStats& st, int win, SampSmem& sm) {
-  double s = 0.0;
-  for (int t = threadIdx.x; t < V; t += SAMP_THREADS) s += (double)expf(z[t] - st.zmax);
-  RasRow rr;
-  rr.sum_full = (float)block_sum_d(s, sm.red_d);
+// R of a row of signed_exp.
+__device__ __forceinline__ float ras_mass(const float* v, const RowStats& st, int win, const SampSmem& sm) {
   float R = 0.f;
   for (int j = 0; j < win; ++j) {  // fixed order
     const int t = sm.rep_ids[j];
-    if (t >= 0 && is_kept(z[t], t, st)) R += expf(z[t] - st.zmax) / st.sum;
+    if (t >= 0 && v[t] > 0.f) R += v[t] / st.sum;
   }
-  rr.R = R;
-  return rr;
+  return R;
 }
-// q(t) of the target's sampler: the (top-k, top-p) softmax, or the repetition-aware mixture.
-__device__ __forceinline__ float q_value(float zz, int t, const RowStats& st, int win, const RasRow& rr,
+// Its share of `sum`, 0 where it is cut off.  (A zero numerator would take the division's slow path, on most of a
+// row under a top-k cut.)
+__device__ __forceinline__ float kept_share(float v, float sum) {
+  const float q = (v > 0.f ? v : 1.f) / sum;
+  return v > 0.f ? q : 0.f;
+}
+
+// q(t) of the target's sampler from signed_exp: the (top-k, top-p) softmax, or the repetition-aware mixture.
+__device__ __forceinline__ float q_value(float v, int t, const RowStats& st, int win, const RasRow& rr,
                                          const SampSmem& sm) {
-  const float e = expf(zz - st.zmax);
-  float q = is_kept(zz, t, st) ? e / st.sum : 0.f;
+  float q = kept_share(v, st.sum);
   if (win > 0) {
     if (q > 0.f && ras_is_rep(sm, win, t)) q = 0.f;
-    q += rr.R * (e / rr.sum_full);
+    q += rr.R * (fabsf(v) / rr.sum_full);
   }
   return q;
 }
@@ -389,109 +606,79 @@ __global__ void __launch_bounds__(SAMP_THREADS)
 verify_sampler_kernel(const float* __restrict__ logits, int V,
                       const int32_t* __restrict__ draft_tokens,
                       const float* __restrict__ draft_probs, const float* __restrict__ uniforms,
-                      int gamma, float inv_t, int top_k, float top_p, float beta, Ras ras, float* row_stats,
-                      int32_t* accept_flags, int32_t* counters, int32_t* __restrict__ accepted_len,
+                      int gamma, float inv_t, int top_k, float top_p, float beta, Ras ras,
+                      int32_t* row_words, int32_t* counters, int32_t* __restrict__ accepted_len,
                       int32_t* __restrict__ next_token, int32_t* status) {
-  tc_pdl_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SampSmem& sm = *reinterpret_cast<SampSmem*>(smem_raw);
   float* z = reinterpret_cast<float*>(smem_raw + sizeof(SampSmem));
-  const int r = blockIdx.x, b = blockIdx.y, R = gamma + 1;
-  const float* lrow = logits + ((size_t)b * R + r) * V;
-  if (threadIdx.x == 0) sm.bad = 0;
-  __syncthreads();
-  int bad = 0;
-  for (int t = threadIdx.x; t < V; t += SAMP_THREADS) {
-    float v = lrow[t];
-    if (!isfinite(v)) bad = 1;
-    z[t] = v * inv_t;
-  }
-  if (bad) sm.bad = 1;
-  __syncthreads();
-  if (sm.bad && threadIdx.x == 0) atomicOr(status, SSD_STATUS_NONFINITE);
-  RowStats st = compute_row_stats(z, V, top_k, top_p, sm);
+  const int tid = threadIdx.x, r = blockIdx.x, b = blockIdx.y, R = gamma + 1;
+  const float* prow = r < gamma ? draft_probs + ((size_t)b * gamma + r) * V : nullptr;
+  clear_bins(sm);
+  if (prow)  // (a hint: whoever writes the row may still be at it)
+    for (int t = tid * 32; t < V; t += SAMP_THREADS * 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(prow + t));
+  tc_pdl_enter();
+  int x = 0;
+  if (tid == 0 && prow) x = draft_tokens[b * gamma + r];
+  const float2 u = make_float2(uniforms[((size_t)b * R + r) * 2], uniforms[((size_t)b * R + r) * 2 + 1]);
+  if (ras.win > 0 && tid >= SAMP_THREADS - 32) ras_window(ras, draft_tokens, gamma, b, r, V, sm);
+  const BinMap map = load_row(logits + ((size_t)b * R + r) * V, V, inv_t, z, sm, status);
+  float px = 0.f;
+  const bool x_ok = x >= 0 && x < V;
+  if (tid == 0 && prow && x_ok) px = prow[x];
   RasRow rr{1.f, 0.f};
-  if (ras.win > 0) {
-    ras_window(ras, draft_tokens, gamma, b, r, V, sm);
-    rr = ras_row(z, V, st, ras.win, sm);
-  }
-  if (threadIdx.x == 0) {
-    int flag = 0;
-    if (r < gamma) {  // Eq. 5: accept x_i iff r_i < min(1, q_i(x_i) / p_i(x_i)) + beta
-      int x = draft_tokens[b * gamma + r];
-      float qx = 0.f, px = 0.f;
-      bool valid = true;  // a draft token or probability that cannot be one is rejected, never accepted
-      if (x < 0 || x >= V) {
-        atomicOr(status, SSD_STATUS_BAD_TOKEN);
+  const RowStats st = compute_row_stats(z, V, top_k, top_p, map, ras.win > 0, &rr.sum_full, sm);
+  if (ras.win > 0) rr.R = ras_mass(z, st, ras.win, sm);
+  int flag = 0;
+  if (tid == 0 && prow) {  // Eq. 5: accept x_i iff r_i < min(1, q_i(x_i) / p_i(x_i)) + beta
+    float qx = 0.f;
+    bool valid = x_ok;  // a draft token or probability that cannot be one is rejected, never accepted
+    if (!x_ok) {
+      atomicOr(status, SSD_STATUS_BAD_TOKEN);
+    } else {
+      qx = q_value(z[x], x, st, ras.win, rr, sm);
+      if (!(px >= 0.f) || !isfinite(px)) {
+        atomicOr(status, SSD_STATUS_BAD_PROB);
         valid = false;
-      } else {
-        qx = q_value(z[x], x, st, ras.win, rr, sm);
-        px = draft_probs[((size_t)b * gamma + r) * V + x];
-        if (!(px >= 0.f) || !isfinite(px)) {
-          atomicOr(status, SSD_STATUS_BAD_PROB);
-          valid = false;
-        }
       }
-      float ratio = px <= qx ? 1.f : qx / px;
-      flag = valid && uniforms[((size_t)b * R + r) * 2] < ratio + beta;
     }
-    float* rs = row_stats + ((size_t)b * R + r) * RS_STRIDE;
-    rs[0] = st.zmax;
-    rs[1] = st.sum;
-    rs[2] = __uint_as_float(st.thr_key);
-    rs[3] = __int_as_float(st.tie_id_max);
-    rs[4] = rr.sum_full;
-    rs[5] = rr.R;
-    accept_flags[b * R + r] = flag;
-    __threadfence();
-    int prev = atomicAdd(&counters[b], 1);
-    sm.last = prev == R - 1;
+    const float ratio = px <= qx ? 1.f : qx / px;
+    flag = valid && u.x < ratio + beta;
   }
-  __syncthreads();
-  if (!sm.last) return;
-  // ---- last CTA of this stream: first rejection, then the one new token ----
-  if (threadIdx.x == 0) {
-    __threadfence();
-    counters[b] = 0;
-    int k = gamma;
-    for (int i = 0; i < gamma; ++i)
-      if (__ldcg(&accept_flags[b * R + i]) == 0) { k = i; break; }
-    sm.k_acc = k;
-  }
-  __syncthreads();
-  const int k = sm.k_acc;
-  const float* rs = row_stats + ((size_t)b * R + k) * RS_STRIDE;
-  RowStats sk;
-  sk.zmax = __ldcg(rs + 0);
-  sk.sum = __ldcg(rs + 1);
-  sk.thr_key = __float_as_uint(__ldcg(rs + 2));
-  sk.tie_id_max = __float_as_int(__ldcg(rs + 3));
-  const RasRow rk{__ldcg(rs + 4), __ldcg(rs + 5)};
-  if (ras.win > 0) ras_window(ras, draft_tokens, gamma, b, k, V, sm);  // row k's repeated ids
-  const float* krow = logits + ((size_t)b * R + k) * V;
-  const float* prow = k < gamma ? draft_probs + ((size_t)b * gamma + k) * V : nullptr;
-  // Eq. 6: w = max(0, q_k - p_k) on a rejection; the bonus row q_{gamma+1} otherwise
-  for (int t = threadIdx.x; t < V; t += SAMP_THREADS) {
-    float zz = krow[t] * inv_t;
-    float q = q_value(zz, t, sk, ras.win, rk, sm);
+  __syncthreads();  // the values above are read: z becomes the weights of the draw
+  // Eq. 6: w = max(0, q_r - p_r), for the case that row r is the first to be rejected; the bonus row q_{gamma+1} otherwise
+#pragma unroll 4
+  for (int t = tid; t < V; t += SAMP_THREADS) {
+    const float q = q_value(z[t], t, st, ras.win, rr, sm);
     z[t] = prow ? fmaxf(0.f, q - prow[t]) : q;
   }
   __syncthreads();
-  const float u = uniforms[((size_t)b * R + k) * 2 + 1];
   double total;
-  int y = block_inverse_cdf(z, V, u, sm, &total);
-  if (y < 0) {  // residual has no mass (numerical corner): draw from q_k itself
-    for (int t = threadIdx.x; t < V; t += SAMP_THREADS) {
-      float zz = krow[t] * inv_t;
-      z[t] = q_value(zz, t, sk, ras.win, rk, sm);
-    }
+  int y = block_inverse_cdf(z, V, u.y, sm, &total);
+  if (y < 0) {  // residual has no mass (numerical corner): draw from q_r itself
+    for (int t = tid; t < V; t += SAMP_THREADS)
+      z[t] = q_value(signed_exp(logits[((size_t)b * R + r) * V + t] * inv_t, t, st, ras.win > 0), t, st, ras.win, rr, sm);
     __syncthreads();
-    y = block_inverse_cdf(z, V, u, sm, &total);
+    y = block_inverse_cdf(z, V, u.y, sm, &total);
     if (y < 0) y = 0;
   }
-  if (threadIdx.x == 0) {
+  // ---- the last CTA of this stream: first rejection, and that row's token ----
+  if (tid >= 32) return;
+  int prev = 0;
+  if (tid == 0) {
+    row_words[b * R + r] = y * 2 + flag;
+    __threadfence();
+    prev = atomicAdd(&counters[b], 1);
+  }
+  if (__shfl_sync(0xffffffffu, prev, 0) != R - 1) return;
+  __threadfence();
+  const int w = tid < R ? __ldcg(&row_words[b * R + tid]) : 1;  // R is at most 16
+  const uint32_t rejected = __ballot_sync(0xffffffffu, tid < gamma && !(w & 1));
+  const int k = rejected ? __ffs(rejected) - 1 : gamma;
+  if (tid == k) {
+    counters[b] = 0;
     accepted_len[b] = k;
-    next_token[b] = y;
+    next_token[b] = w >> 1;
   }
 }
 
@@ -499,7 +686,7 @@ cudaError_t launch_verify_sampler(const float* logits, int V, const int32_t* dra
                                   const float* draft_probs, const float* uniforms, int B,
                                   int gamma, float inv_temperature, int top_k, float top_p, float beta,
                                   int ras_window, float ras_tau, const int32_t* recent_tokens,
-                                  float* row_stats, int32_t* accept_flags, int32_t* counters,
+                                  int32_t* row_words, int32_t* counters,
                                   int32_t* accepted_len, int32_t* next_token, int32_t* status,
                                   cudaStream_t st) {
   Ras ras{0, 0.f, nullptr};
@@ -508,7 +695,7 @@ cudaError_t launch_verify_sampler(const float* logits, int V, const int32_t* dra
     ras = Ras{ras_window, (float)ras_window * ras_tau, recent_tokens};
   }
   size_t smem = sizeof(SampSmem) + (size_t)V * sizeof(float);
-  if (smem > 200 * 1024) return cudaErrorInvalidValue;
+  if (smem > 227 * 1024) return cudaErrorInvalidValue;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(verify_sampler_kernel,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -516,7 +703,7 @@ cudaError_t launch_verify_sampler(const float* logits, int V, const int32_t* dra
   }
   dim3 grid(gamma + 1, B);
   tc_launch_pdl(verify_sampler_kernel, grid, dim3(SAMP_THREADS), smem, st, logits, V, draft_tokens, draft_probs,
-                uniforms, gamma, inv_temperature, top_k, top_p, beta, ras, row_stats, accept_flags, counters,
+                uniforms, gamma, inv_temperature, top_k, top_p, beta, ras, row_words, counters,
                 accepted_len, next_token, status);
   count_launch();
   return cudaGetLastError();
@@ -529,32 +716,25 @@ draft_sampler_kernel(const float* __restrict__ logits, int ld_logits, int V,
                      const float* __restrict__ uniform, float inv_t, int top_k, float top_p,
                      int32_t* __restrict__ out_token, int tok_stride, float* __restrict__ out_prob,
                      size_t prob_stride, int32_t* pending, int32_t* status) {
-  tc_pdl_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SampSmem& sm = *reinterpret_cast<SampSmem*>(smem_raw);
   float* z = reinterpret_cast<float*>(smem_raw + sizeof(SampSmem));
   const int b = blockIdx.x;
-  const float* lrow = logits + (size_t)b * ld_logits;
-  if (threadIdx.x == 0) sm.bad = 0;
-  __syncthreads();
-  int bad = 0;
-  for (int t = threadIdx.x; t < V; t += SAMP_THREADS) {
-    float v = lrow[t];
-    if (!isfinite(v)) bad = 1;
-    z[t] = v * inv_t;
-  }
-  if (bad) sm.bad = 1;
-  __syncthreads();
-  if (sm.bad && threadIdx.x == 0) atomicOr(status, SSD_STATUS_NONFINITE);
-  RowStats st = compute_row_stats(z, V, top_k, top_p, sm);
-  for (int t = threadIdx.x; t < V; t += SAMP_THREADS) {
-    float p = is_kept(z[t], t, st) ? expf(z[t] - st.zmax) / st.sum : 0.f;
+  clear_bins(sm);
+  tc_pdl_enter();
+  const float u = uniform[b];
+  const BinMap map = load_row(logits + (size_t)b * ld_logits, V, inv_t, z, sm, status);
+  float sum_full;
+  const RowStats st = compute_row_stats(z, V, top_k, top_p, map, false, &sum_full, sm);
+#pragma unroll 4
+  for (int t = threadIdx.x; t < V; t += SAMP_THREADS) {  // each thread's own elements of z: no barrier before
+    const float p = kept_share(z[t], st.sum);
     z[t] = p;
     out_prob[(size_t)b * prob_stride + t] = p;
   }
   __syncthreads();
   double total;
-  int y = block_inverse_cdf(z, V, uniform[b], sm, &total);
+  int y = block_inverse_cdf(z, V, u, sm, &total);
   if (y < 0) y = 0;
   if (threadIdx.x == 0) {
     out_token[(size_t)b * tok_stride] = y;
@@ -568,7 +748,7 @@ cudaError_t launch_draft_sampler(const float* logits, int ld_logits, int V, cons
                                  size_t prob_stride, int32_t* pending, int32_t* status,
                                  cudaStream_t st) {
   size_t smem = sizeof(SampSmem) + (size_t)V * sizeof(float);
-  if (smem > 200 * 1024) return cudaErrorInvalidValue;
+  if (smem > 227 * 1024) return cudaErrorInvalidValue;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(draft_sampler_kernel,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -618,21 +798,19 @@ void launch_kv_commit(int32_t* len, int32_t* pending, const int32_t* accepted_le
 // whose memory pool is fixed at start-up, or a plug-in that is handed device pointers by its host
 // process and owns none.  ssd_verify needs a workspace such callers cannot provide.  This entry
 // point runs the same fused acceptance kernel on logits the caller already has, and keeps the
-// kernel's scratch (eight statistics words and one flag per row, one counter per stream, one status
-// word) in the fixed device array below instead.
+// kernel's scratch (one word per row, one counter per stream, one status word) in the fixed device array below instead.
 namespace {
 
 constexpr int NOALLOC_MAX_STREAMS = 256;  // streams per call
 constexpr int NOALLOC_MAX_ROWS = ssd::R_MAX;  // gamma + 1 <= 16
 
 struct NoAllocScratch {
-  float row_stats[NOALLOC_MAX_STREAMS * NOALLOC_MAX_ROWS * ssd::RS_STRIDE];
-  int32_t accept_flags[NOALLOC_MAX_STREAMS * NOALLOC_MAX_ROWS];
+  int32_t row_words[NOALLOC_MAX_STREAMS * NOALLOC_MAX_ROWS];
   int32_t counters[NOALLOC_MAX_STREAMS];
   int32_t status;
 };
 
-// About 148 KB, resident on every GPU that loads the library until the process exits.  In host
+// About 17 KB, resident on every GPU that loads the library until the process exits.  In host
 // code this name is only a handle for cudaGetSymbolAddress, never a device address.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(NoAllocScratch)];
 
@@ -683,7 +861,7 @@ extern "C" int ssd_accept_noalloc(const float* dev_logits, const int32_t* dev_dr
   e = ssd::launch_verify_sampler(dev_logits, vocab, dev_draft_tokens, dev_draft_probs, dev_uniforms,
                                  batch, params->gamma, 1.0f / params->temperature, params->top_k,
                                  params->top_p, params->beta, params->ras_window, params->ras_tau,
-                                 params->dev_recent_tokens, sc->row_stats, sc->accept_flags, sc->counters,
+                                 params->dev_recent_tokens, sc->row_words, sc->counters,
                                  dev_accepted_len, dev_next_token, &sc->status, st);
   if (e != cudaSuccess) return ssd::report_cuda_error(e, "ssd_accept_noalloc: launch");
   return SSD_OK;
