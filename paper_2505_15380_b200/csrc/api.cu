@@ -463,8 +463,8 @@ int forward_chain(const ssd_model* m, ssd_streams* s, RowMap rm, const int32_t* 
   return SSD_OK;
 }
 
-int forward_tc(const ssd_model* m, ssd_streams* s, RowMap rm, float* logits_out, cudaStream_t st,
-               const PrefillSegs* segs = nullptr) {
+int forward_tc(const ssd_model* m, ssd_streams* s, RowMap rm, const int32_t* draft_tokens, float* logits_out,
+               cudaStream_t st, const PrefillSegs* segs = nullptr) {
   const ssd_model_config& c = m->cfg;
   const int M = row_count(rm), Mpad = tc_round16(M), d = c.d_model;
   const int qd = c.n_q_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim, F = c.d_ffn, nq = qd + 2 * kvd;
@@ -485,8 +485,8 @@ int forward_tc(const ssd_model* m, ssd_streams* s, RowMap rm, float* logits_out,
   else if (s->paged)  // every stream of this forward owns pages for the rows it is about to append
     launch_page_ensure(s->len, rm, s->page_table, s->pages_used, s->free_stack, s->free_top, s->max_pages,
                        s->status, st);
-  launch_embed(1, m->embed, c.vocab_out + c.vocab_text, d, s->row_ids, M, s->h, s->status, st);
-  launch_rope_table(s->len, rm, m->inv_freq, c.head_dim / 2, s->rope_cs, st);
+  launch_embed(1, m->embed, c.vocab_out + c.vocab_text, d, draft_tokens ? nullptr : s->row_ids, s->pending, draft_tokens,
+               s->len, rm, m->inv_freq, c.head_dim / 2, s->h, s->rope_cs, s->status, st);
   // pair kernel: whether a projection's slices are added within its CTAs, or written out one by one
   const bool in_qkv = pairs && tc_prefill_groups(nq, M, ks_qkv, n_sm) == 1, in_o = pairs && tc_prefill_groups(d, M, ks_o, n_sm) == 1,
              in_d = pairs && tc_prefill_groups(d, M, ks_d, n_sm) == 1;
@@ -538,40 +538,50 @@ int forward_tc(const ssd_model* m, ssd_streams* s, RowMap rm, float* logits_out,
   return SSD_OK;
 }
 
-int forward(const ssd_model* m, ssd_streams* s, RowMap rm, float* logits_out, cudaStream_t st) {
-  if (use_chain(m, s, rm)) return forward_chain(m, s, rm, nullptr, logits_out, st);
-  if (s->paged) return forward_tc(m, s, rm, logits_out, st);
-  if (use_fast(m, s, rm)) return forward_fast(m, s, rm, s->row_ids, nullptr, logits_out, st);
-  if (use_tc(m, s, rm)) return forward_tc(m, s, rm, logits_out, st);
+// Ids: s->row_ids, or (draft_tokens given) those of a verify step.
+int forward(const ssd_model* m, ssd_streams* s, RowMap rm, const int32_t* draft_tokens, float* logits_out, cudaStream_t st) {
+  if (use_chain(m, s, rm)) return forward_chain(m, s, rm, draft_tokens, logits_out, st);
+  if (s->paged) return forward_tc(m, s, rm, draft_tokens, logits_out, st);
+  if (use_fast(m, s, rm)) return forward_fast(m, s, rm, draft_tokens ? nullptr : s->row_ids, draft_tokens, logits_out, st);
+  if (use_tc(m, s, rm)) return forward_tc(m, s, rm, draft_tokens, logits_out, st);
   const ssd_model_config& c = m->cfg;
-  const int dt = c.weight_dtype, M = rm.nb * rm.R, d = c.d_model;
-  const int qd = c.n_q_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim, F = c.d_ffn;
-  launch_embed(dt, m->embed, c.vocab_out + c.vocab_text, d, s->row_ids, M, s->h, s->status, st);
-  launch_rope_table(s->len, rm, m->inv_freq, c.head_dim / 2, s->rope_cs, st);
+  const int dt = c.weight_dtype, M = rm.nb * rm.R, d = c.d_model, hd = c.head_dim;
+  const int qd = c.n_q_heads * hd, kvd = c.n_kv_heads * hd, F = c.d_ffn;
+  launch_embed(dt, m->embed, c.vocab_out + c.vocab_text, d, draft_tokens ? nullptr : s->row_ids, s->pending, draft_tokens,
+               s->len, rm, m->inv_freq, hd / 2, s->h, s->rope_cs, s->status, st);
+  auto normed = [&](const void* gain) {  // RMSNorm as the projection's CTAs stage the rows, or ahead of it
+    if (d <= GEMM_FUSED_K) return SimtSrc{s->h, d, gain, c.rms_eps};
+    launch_rmsnorm(dt, s->h, gain, s->xn, M, d, c.rms_eps, st);
+    return SimtSrc{s->xn, d};
+  };
+  SimtSrc merged{s->attn_out, qd};
+  // Every CTA of the O projection reads the partials of its 8 rows: up to 64 KB that costs less than a launch.
+  const bool merge_in_o = (long)s->nsplit_max * qd <= 2048;
+  if (merge_in_o) {
+    merged.part = s->part;
+    merged.len = s->len;
+    merged.rm = rm;
+    merged.cap = s->cap;
+    merged.Hq = c.n_q_heads;
+    merged.hd = hd;
+    merged.nsplit_max = s->nsplit_max;
+  }
   for (int l = 0; l < c.n_layers; ++l) {
     const LayerW& w = m->layers[l];
     void* kv_layer = s->kv + (size_t)l * s->kv_layer_elems * s->el;
-    launch_rmsnorm(dt, s->h, w.norm1, s->xn, M, d, c.rms_eps, st);
-    SSD_CUDA(launch_gemm_simt(dt, EPI_STORE_F32, s->xn, d, w.w_qkv, w.b_qkv, s->qkv,
-                              qd + 2 * kvd, M, qd + 2 * kvd, d, st));
-    launch_qkv_post(dt, s->qkv, s->rope_cs, s->qrot, kv_layer, s->len, rm, s->cap, c.n_q_heads,
-                    c.n_kv_heads, c.head_dim, s->status, st);
-    SSD_CUDA(launch_attention_simt(dt, s->qrot, kv_layer, s->len, rm, s->cap, c.n_q_heads,
-                                   c.n_kv_heads, c.head_dim, s->part, s->nsplit_max, s->attn_out,
-                                   st));
-    SSD_CUDA(launch_gemm_simt(dt, EPI_RESIDUAL, s->attn_out, qd, w.w_o, nullptr, s->h, d,
-                              M, d, qd, st));
-    launch_rmsnorm(dt, s->h, w.norm2, s->xn, M, d, c.rms_eps, st);
-    SSD_CUDA(launch_gemm_simt(dt, EPI_SWIGLU, s->xn, d, w.w_gu, nullptr, s->act, F, M,
-                              2 * F, d, st));
-    SSD_CUDA(launch_gemm_simt(dt, EPI_RESIDUAL, s->act, F, w.w_d, nullptr, s->h, d, M, d,
-                              F, st));
+    SSD_CUDA(launch_gemm_simt(dt, EPI_STORE_F32, normed(w.norm1), w.w_qkv, w.b_qkv, s->qkv, qd + 2 * kvd, M,
+                              qd + 2 * kvd, d, st));
+    SSD_CUDA(launch_attention_simt(dt, s->qkv, s->rope_cs, kv_layer, s->len, rm, s->cap, c.n_q_heads, c.n_kv_heads, hd,
+                                   s->part, s->nsplit_max, s->status, st));
+    if (!merge_in_o)
+      SSD_CUDA(launch_attention_merge(s->part, s->len, rm, s->cap, c.n_q_heads, hd, s->nsplit_max, s->attn_out, st));
+    SSD_CUDA(launch_gemm_simt(dt, EPI_RESIDUAL, merged, w.w_o, nullptr, s->h, d, M, d, qd, st));
+    SSD_CUDA(launch_gemm_simt(dt, EPI_SWIGLU, normed(w.norm2), w.w_gu, nullptr, s->act, F, M, 2 * F, d, st));
+    SSD_CUDA(launch_gemm_simt(dt, EPI_RESIDUAL, SimtSrc{s->act, F}, w.w_d, nullptr, s->h, d, M, d, F, st));
   }
-  if (logits_out) {
-    launch_rmsnorm(dt, s->h, m->norm_f, s->xn, M, d, c.rms_eps, st);
-    SSD_CUDA(launch_gemm_simt(dt, EPI_STORE_F32, s->xn, d, m->head, nullptr, logits_out,
-                              c.vocab_out, M, c.vocab_out, d, st));
-  }
+  if (logits_out)
+    SSD_CUDA(launch_gemm_simt(dt, EPI_STORE_F32, normed(m->norm_f), m->head, nullptr, logits_out, c.vocab_out, M,
+                              c.vocab_out, d, st));
   SSD_CUDA(cudaGetLastError());
   return SSD_OK;
 }
@@ -617,7 +627,7 @@ int prefill_tc(ssd_model* m, ssd_streams* s, const int32_t* ids, const int32_t* 
       int rc;
       if (P.n == 1 && use_fast(m, s, one)) {
         SSD_CUDA(cudaMemcpyAsync(s->row_ids, ids + P.s[0].src, (size_t)P.n_rows * 4, cudaMemcpyDeviceToDevice, st));
-        rc = forward(m, s, one, nullptr, st);
+        rc = forward(m, s, one, nullptr, nullptr, st);
       } else {
         RowMap rm{0, 0, 1};
         rm.rows = s->tc_rowmap;
@@ -625,7 +635,7 @@ int prefill_tc(ssd_model* m, ssd_streams* s, const int32_t* ids, const int32_t* 
         rm.n_rows = P.n_rows;
         rm.n_tiles = P.n_tiles;
         launch_prefill_stage(P, ids, s->row_ids, s->tc_rowmap, s->tc_tiles, st);
-        rc = forward_tc(m, s, rm, nullptr, st, &P);
+        rc = forward_tc(m, s, rm, nullptr, nullptr, st, &P);
       }
       if (rc != SSD_OK) return rc;
     }
@@ -649,7 +659,7 @@ int draft_step_impl(ssd_model* draft, ssd_streams* ds, const int32_t* ids, int n
   } else {
     SSD_CUDA(cudaMemcpyAsync(ds->row_ids, ids ? ids : ds->pending, (size_t)ds->B * n_in * 4,
                              cudaMemcpyDeviceToDevice, st));
-    rc = forward(draft, ds, rm, ds->logits, st);
+    rc = forward(draft, ds, rm, nullptr, ds->logits, st);
   }
   if (rc != SSD_OK) return rc;
   launch_advance_all(ds->len, ds->B, n_in, ds->cap, ds->status, st);
@@ -1130,10 +1140,7 @@ int ssd_forward(ssd_model* model, ssd_streams* s, const int32_t* dev_draft_token
   if (gamma < 1 || gamma > s->max_gamma) return SSD_ERR_BAD_GAMMA;
   cudaStream_t st = (cudaStream_t)stream;
   const RowMap rm{0, s->B, gamma + 1};
-  if (use_fast(model, s, rm)) return forward_fast(model, s, rm, nullptr, dev_draft_tokens, dev_logits, st);
-  if (use_chain(model, s, rm)) return forward_chain(model, s, rm, dev_draft_tokens, dev_logits, st);
-  launch_gather_verify_ids(s->pending, dev_draft_tokens, gamma, s->B, s->row_ids, st);
-  return forward(model, s, rm, dev_logits, st);
+  return forward(model, s, rm, dev_draft_tokens, dev_logits, st);
 }
 
 int ssd_streams_set_attention_kernel(ssd_streams* s, int32_t which) {
@@ -1216,7 +1223,7 @@ int ssd_prefill(ssd_model* m, ssd_streams* s, const int32_t* dev_ids, const int3
     for (int done = 0; done < n - 1; done += chunk) {
       int rows = n - 1 - done < chunk ? n - 1 - done : chunk;
       SSD_CUDA(cudaMemcpyAsync(s->row_ids, ids + done, rows * 4, cudaMemcpyDeviceToDevice, st));
-      int rc = forward(m, s, RowMap{b, 1, rows}, nullptr, st);
+      int rc = forward(m, s, RowMap{b, 1, rows}, nullptr, nullptr, st);
       if (rc != SSD_OK) return rc;
       launch_advance_len(s->len, s->pending, b, rows, ids, -1, st);
     }
@@ -1306,11 +1313,8 @@ int verify_impl(ssd_model* target, ssd_streams* s, const int32_t* dev_draft_toke
   int rc;
   if (use_fast(target, s, rm, whole_nucleus(params, target->cfg.vocab_out))) {
     rc = forward_fast(target, s, rm, nullptr, dev_draft_tokens, logits, st);
-  } else if (use_chain(target, s, rm)) {
-    rc = forward_chain(target, s, rm, dev_draft_tokens, logits, st);
   } else {
-    launch_gather_verify_ids(s->pending, dev_draft_tokens, gamma, s->B, s->row_ids, st);
-    rc = forward(target, s, rm, logits, st);
+    rc = forward(target, s, rm, dev_draft_tokens, logits, st);
   }
   if (rc != SSD_OK) return rc;
   if (upload) {

@@ -13,17 +13,12 @@ int report_cuda_error(cudaError_t e, const char* what);
 enum Epilogue { EPI_STORE_F32 = 0, EPI_RESIDUAL = 1, EPI_SWIGLU = 2 };
 
 // elementwise.cu
-void launch_gather_verify_ids(const int32_t* pending, const int32_t* draft_tokens, int gamma,
-                              int B, int32_t* row_ids, cudaStream_t st);
-void launch_embed(int dtype, const void* table, int vocab_in, int d, const int32_t* row_ids, int M,
-                  float* h, int32_t* status, cudaStream_t st);
-void launch_rope_table(const int32_t* len, RowMap rm, const double* inv_freq, int half, float* cs,
-                       cudaStream_t st);
+// The rows entering a forward; row_ids null: those of a verify step, from pending and draft.
+void launch_embed(int dtype, const void* table, int vocab_in, int d, const int32_t* row_ids, const int32_t* pending,
+                  const int32_t* draft, const int32_t* len, RowMap rm, const double* inv_freq, int half, float* h,
+                  float* cs, int32_t* status, cudaStream_t st);
 void launch_rmsnorm(int dtype, const float* h, const void* gain, float* out, int M, int d, float eps,
                     cudaStream_t st);
-void launch_qkv_post(int dtype, const float* qkv, const float* cs, float* qrot, void* kv_layer,
-                     const int32_t* len, RowMap rm, int cap, int Hq, int Hkv, int hd,
-                     int32_t* status, cudaStream_t st);
 void launch_prefill_stage(const PrefillSegs& segs, const int32_t* ids, int32_t* row_ids, int2* rows, int4* tiles,
                           cudaStream_t st);
 void launch_prefill_advance(const PrefillSegs& segs, const int32_t* ids, int32_t* len, int32_t* pending,
@@ -40,14 +35,29 @@ void launch_advance_all(int32_t* len, int B, int add, int cap, int32_t* status, 
 //   EPI_RESIDUAL  : C[m, n]  += acc
 //   EPI_SWIGLU    : C[m, n/2] = silu(acc[2j]) * acc[2j+1]           (W rows interleaved g,u)
 // Activations and outputs are fp32; `dtype` is the storage type of W and bias.
-cudaError_t launch_gemm_simt(int dtype, int epi, const float* A, int lda, const void* W,
-                             const void* bias, float* C, int ldc, int M, int N, int K,
-                             cudaStream_t st);
+// A is `src.a` [M, lda], or
+//   src.gain  : its rows after RMSNorm                              (K <= GEMM_FUSED_K)
+//   src.part  : the attention's partials of the rows' heads, merged (K <= GEMM_FUSED_K)
+constexpr int GEMM_FUSED_K = 2048;
+struct SimtSrc {
+  const float* a;
+  int lda;
+  const void* gain = nullptr;  // storage type of W
+  float eps = 0.f;
+  const float* part = nullptr;
+  const int32_t* len = nullptr;
+  RowMap rm{};
+  int cap = 0, Hq = 0, hd = 0, nsplit_max = 0;
+};
+cudaError_t launch_gemm_simt(int dtype, int epi, const SimtSrc& src, const void* W, const void* bias, float* C, int ldc,
+                             int M, int N, int K, cudaStream_t st);
 
-// attention_simt.cu
-cudaError_t launch_attention_simt(int dtype, const float* qrot, const void* kv_layer,
-                                  const int32_t* len, RowMap rm, int cap, int Hq, int Hkv, int hd,
-                                  float* part, int nsplit_max, float* out, cudaStream_t st);
+// attention_simt.cu: rotates q and the new keys, appends K/V to the cache, leaves partials per split
+cudaError_t launch_attention_simt(int dtype, const float* qkv, const float* cs, void* kv_layer, const int32_t* len,
+                                  RowMap rm, int cap, int Hq, int Hkv, int hd, float* part, int nsplit_max,
+                                  int32_t* status, cudaStream_t st);
+cudaError_t launch_attention_merge(const float* part, const int32_t* len, RowMap rm, int cap, int Hq, int hd,
+                                   int nsplit_max, float* out, cudaStream_t st);
 
 // sampler.cu
 cudaError_t launch_verify_sampler(const float* logits, int V, const int32_t* draft_tokens,
