@@ -323,7 +323,7 @@ int ssd_iteration(ssd_model* target, ssd_streams* target_streams, ssd_model* dra
  * bonus draw of Eq. 6 exactly as ssd_verify does, and writes the same two outputs.
  *   in  dev_logits float [batch, gamma+1, vocab]; dev_draft_tokens, dev_draft_probs, dev_uniforms
  *       as in ssd_verify;  out dev_accepted_len, dev_next_token int32 [batch].
- * The kernel's scratch lives in a fixed array inside the library (about 148 KB, held by every GPU
+ * The kernel's scratch lives in a fixed array inside the library (about 17 KB, held by every GPU
  * that loads the library until the process exits), sized for at most 256 streams and
  * gamma + 1 <= 16 rows: larger batches return SSD_ERR_TOO_SMALL, larger gamma SSD_ERR_BAD_GAMMA.
  * No cudaMalloc / cudaFree or allocating library routine is called.  The first call on a device

@@ -588,46 +588,32 @@ int forward(const ssd_model* m, ssd_streams* s, RowMap rm, const int32_t* draft_
 
 // Prefill on the tensor-core path: the prompts' rows, all streams one after the other, are cut into
 // equal chunks of at most tc_rows rows; a chunk is one forward whose rows may belong to several
-// streams (causal within each).  A last chunk of few rows of one stream is the persistent kernel's.
+// streams (causal within each).  A prompt that fits the persistent kernel takes it by itself, whoever
+// joins beside it: what a prompt leaves in the cache does not depend on its neighbours.
 int prefill_tc(ssd_model* m, ssd_streams* s, const int32_t* ids, const int32_t* off, cudaStream_t st) {
   const int G = m->cfg.n_q_heads / m->cfg.n_kv_heads;
-  long long left = 0;
-  for (int b = 0; b < s->B; ++b) left += std::max(off[b + 1] - off[b] - 1, 0);
-  const long long n_chunks = std::max<long long>((left + s->tc_rows - 1) / s->tc_rows, 1);
-  const int target = std::min((int)align_up((size_t)((left + n_chunks - 1) / n_chunks), 16), s->tc_rows);
-  int b = 0, done = 0;  // next stream, rows of it already taken
-  while (b < s->B) {
-    PrefillSegs P{};
-    P.tile_rows = 64 / G;
-    while (b < s->B && P.n < PREFILL_SEGS) {
-      const int n = off[b + 1] - off[b];
-      if (n == 0) {  // takes no part
-        ++b;
-        continue;
-      }
-      const int count = std::min(n - 1 - done, target - P.n_rows);
-      if (count == 0 && done < n - 1) break;  // the chunk is full
-      const bool ends = done + count == n - 1;
-      P.s[P.n].stream = b;
-      P.s[P.n].src = off[b] + done;
-      P.s[P.n].count = count;
-      P.s[P.n].m0 = P.n_rows;
-      P.s[P.n].tile0 = P.n_tiles;
-      P.s[P.n].pend_src = ends ? off[b] + n - 1 : -1;
-      ++P.n;
-      P.n_rows += count;
-      P.n_tiles += (count + P.tile_rows - 1) / P.tile_rows;
-      done = ends ? 0 : done + count;
-      if (ends) ++b;
-      else break;
-    }
-    if (P.n == 0) break;
+  auto alone = [&](int b) {
+    const int rows = off[b + 1] - off[b] - 1;
+    return rows > 0 && rows <= FAST_MAX_T && use_fast(m, s, RowMap{b, 1, rows});
+  };
+  auto add = [&](PrefillSegs& P, int b, int done, int count) {  // `count` rows of stream b, from `done` on
+    const int n = off[b + 1] - off[b];
+    P.s[P.n].stream = b;
+    P.s[P.n].src = off[b] + done;
+    P.s[P.n].count = count;
+    P.s[P.n].m0 = P.n_rows;
+    P.s[P.n].tile0 = P.n_tiles;
+    P.s[P.n].pend_src = done + count == n - 1 ? off[b] + n - 1 : -1;
+    ++P.n;
+    P.n_rows += count;
+    P.n_tiles += (count + P.tile_rows - 1) / P.tile_rows;
+  };
+  auto run = [&](const PrefillSegs& P) -> int {
     if (P.n_rows > 0) {
       const RowMap one{P.s[0].stream, 1, P.n_rows};
       int rc;
       if (P.n == 1 && use_fast(m, s, one)) {
-        SSD_CUDA(cudaMemcpyAsync(s->row_ids, ids + P.s[0].src, (size_t)P.n_rows * 4, cudaMemcpyDeviceToDevice, st));
-        rc = forward(m, s, one, nullptr, nullptr, st);
+        rc = forward_fast(m, s, one, ids + P.s[0].src, nullptr, nullptr, st);
       } else {
         RowMap rm{0, 0, 1};
         rm.rows = s->tc_rowmap;
@@ -640,6 +626,43 @@ int prefill_tc(ssd_model* m, ssd_streams* s, const int32_t* ids, const int32_t* 
       if (rc != SSD_OK) return rc;
     }
     launch_prefill_advance(P, ids, s->len, s->pending, st);
+    return SSD_OK;
+  };
+  long long left = 0;
+  for (int b = 0; b < s->B; ++b) {
+    if (!alone(b)) {
+      left += std::max(off[b + 1] - off[b] - 1, 0);
+      continue;
+    }
+    PrefillSegs P{};
+    P.tile_rows = 64 / G;
+    add(P, b, 0, off[b + 1] - off[b] - 1);
+    const int rc = run(P);
+    if (rc != SSD_OK) return rc;
+  }
+  const long long n_chunks = std::max<long long>((left + s->tc_rows - 1) / s->tc_rows, 1);
+  const int target = std::min((int)align_up((size_t)((left + n_chunks - 1) / n_chunks), 16), s->tc_rows);
+  int b = 0, done = 0;  // next stream, rows of it already taken
+  while (b < s->B) {
+    PrefillSegs P{};
+    P.tile_rows = 64 / G;
+    while (b < s->B && P.n < PREFILL_SEGS) {
+      const int n = off[b + 1] - off[b];
+      if (n == 0 || alone(b)) {  // takes no part
+        ++b;
+        continue;
+      }
+      const int count = std::min(n - 1 - done, target - P.n_rows);
+      if (count == 0 && done < n - 1) break;  // the chunk is full
+      add(P, b, done, count);
+      done += count;
+      if (done < n - 1) break;
+      done = 0;
+      ++b;
+    }
+    if (P.n == 0) break;
+    const int rc = run(P);
+    if (rc != SSD_OK) return rc;
   }
   SSD_CUDA(cudaGetLastError());
   return SSD_OK;
@@ -1090,7 +1113,6 @@ void ssd_streams_destroy(ssd_streams* s) {
   if (!s) return;
   if (s->copy_stream) {
     cudaStreamDestroy(s->copy_stream);
-    cudaEventDestroy(s->ev_free);
     cudaEventDestroy(s->ev_probs);
     if (s->h_stage) cudaFreeHost(s->h_stage);
   }
@@ -1299,7 +1321,6 @@ struct ProbsUpload {
   const void* host_src;
   void* dev_dst;
   size_t bytes;
-  cudaEvent_t dst_free;  // already recorded on the main stream: earlier readers of dev_dst are done
   cudaEvent_t ready;
 };
 
@@ -1318,7 +1339,6 @@ int verify_impl(ssd_model* target, ssd_streams* s, const int32_t* dev_draft_toke
   }
   if (rc != SSD_OK) return rc;
   if (upload) {
-    SSD_CUDA(cudaStreamWaitEvent(upload->side, upload->dst_free, 0));
     SSD_CUDA(cudaMemcpyAsync(upload->dev_dst, upload->host_src, upload->bytes, cudaMemcpyHostToDevice, upload->side));
     SSD_CUDA(cudaEventRecord(upload->ready, upload->side));
     SSD_CUDA(cudaStreamWaitEvent(st, upload->ready, 0));
@@ -1375,28 +1395,27 @@ int ssd_verify_host(ssd_model* target, ssd_streams* s, const int32_t* host_draft
   const size_t B = s->B, g = params->gamma, V = s->cfg.vocab_out;
   if (!s->copy_stream) {  // side stream and events of the overlapped upload, made on first use
     SSD_CUDA(cudaStreamCreateWithFlags(&s->copy_stream, cudaStreamNonBlocking));
-    SSD_CUDA(cudaEventCreateWithFlags(&s->ev_free, cudaEventDisableTiming));
     SSD_CUDA(cudaEventCreateWithFlags(&s->ev_probs, cudaEventDisableTiming));
     // pinned host staging for the small inputs and the two result arrays (host memory, not device)
     s->h_stage_in = (size_t)((char*)s->st_uni - (char*)s->st_tokens) + (size_t)s->max_rows * 2 * 4;
     SSD_CUDA(cudaHostAlloc((void**)&s->h_stage, s->h_stage_in + 2 * B * 4, cudaHostAllocDefault));
   }
   // The draft rows are by far the largest input and only the acceptance kernel reads them: they
-  // travel on the side stream (after whatever still reads the staging buffer on `stream`), and
-  // that copy is enqueued once the forward has been launched; the small inputs go ahead.
-  SSD_CUDA(cudaEventRecord(s->ev_free, st));
-  const ProbsUpload upload{s->copy_stream, host_draft_probs, s->st_probs, B * g * V * 4, s->ev_free, s->ev_probs};
-  // tokens and uniforms: gathered in the pinned staging buffer (a few hundred bytes), one copy
+  // travel on the side stream, and that copy is enqueued once the forward has been launched.  (Whoever
+  // read their place before was waited for at the end of the last call.)
+  const ProbsUpload upload{s->copy_stream, host_draft_probs, s->st_probs, B * g * V * 4, s->ev_probs};
+  // Tokens and uniforms go through the pinned staging buffer (a few hundred bytes), from which a kernel fetches
+  // them, and the commit writes k and y back to it: a copy in front and one behind took 5 us each.
   const size_t uni_off = (size_t)((char*)s->st_uni - (char*)s->st_tokens), uni_bytes = B * (g + 1) * 2 * 4;
   memcpy(s->h_stage, host_draft_tokens, B * g * 4);
   memcpy(s->h_stage + uni_off, host_uniforms, uni_bytes);
-  SSD_CUDA(cudaMemcpyAsync(s->st_tokens, s->h_stage, uni_off + uni_bytes, cudaMemcpyHostToDevice, st));
+  launch_fetch_words((const uint32_t*)s->h_stage, (uint32_t*)s->st_tokens, (int)((uni_off + uni_bytes) / 4), st);
   rc = verify_impl(target, s, s->st_tokens, s->st_probs, s->st_uni, params, s->st_k, s->st_y, nullptr, st, &upload);
   if (rc != SSD_OK) return rc;
-  rc = ssd_kv_commit(s, s->st_k, s->st_y, stream);
-  if (rc != SSD_OK) return rc;
-  char* h_out = s->h_stage + s->h_stage_in;  // [k | y] come back with one copy
-  SSD_CUDA(cudaMemcpyAsync(h_out, s->st_k, 2 * B * 4, cudaMemcpyDeviceToHost, st));
+  char* h_out = s->h_stage + s->h_stage_in;  // [k | y]
+  launch_kv_commit(s->len, s->pending, s->st_k, s->st_y, s->B, s->cap, s->max_gamma, s->status, st, (int32_t*)h_out);
+  release_pages(s, st);
+  SSD_CUDA(cudaGetLastError());
   SSD_CUDA(cudaStreamSynchronize(st));
   memcpy(host_accepted_len, h_out, B * 4);
   memcpy(host_next_token, h_out + B * 4, B * 4);

@@ -164,9 +164,9 @@ struct ssd_streams {
   int4* tc_tiles;
   uint8_t *tc_xa, *tc_xattn, *tc_xact;
   float* tc_part;
-  // host-buffer entry: side stream for the upload of the draft rows, and its two events
+  // host-buffer entry: side stream for the upload of the draft rows, and its event
   cudaStream_t copy_stream = nullptr;
-  cudaEvent_t ev_free = nullptr, ev_probs = nullptr;
+  cudaEvent_t ev_probs = nullptr;
   char* h_stage = nullptr;  // pinned host staging of that entry: [tokens | uniforms] then [k | y]
   size_t h_stage_in = 0;
   int split_act;     // persistent kernel: activations as bf16 hi + lo pairs (1) or plain bf16 (0)

@@ -142,6 +142,18 @@ void launch_prefill_advance(const PrefillSegs& segs, const int32_t* ids, int32_t
   count_launch();
 }
 
+__global__ void fetch_words_kernel(const uint32_t* __restrict__ host, uint32_t* __restrict__ dst, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t v = i < n ? host[i] : 0u;  // ahead of the wait: nothing on the device writes it
+  tc_pdl_enter();
+  if (i < n) dst[i] = v;
+}
+
+void launch_fetch_words(const uint32_t* host, uint32_t* dst, int n, cudaStream_t st) {
+  tc_launch_pdl(fetch_words_kernel, dim3((n + 127) / 128), dim3(128), 0, st, host, dst, n);
+  count_launch();
+}
+
 // O(1) rollback from device arrays: len[b] = src_len[b] (clamped to the capacity).
 __global__ void kv_restore_kernel(int32_t* len, int32_t* pending, const int32_t* src_len,
                                   const int32_t* src_pending, int B, int cap) {

@@ -1171,19 +1171,22 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) fast_forward_kernel(const __g
   uint8_t* uni = smem + P.union_off;
   int n_trace = 0;
 
-  // a launch that failed earlier leaves the barrier words unusable: refuse to run on them
-  if (ld_acquire_u32(P.epoch_base + 1) != 0u) {
-    if (cta == 0 && tid == 0) atomicOr(P.status, SSD_STATUS_TIMEOUT);
-    return;
-  }
+  // What the set-up reads, all requested at once: one dependent trip to L2 after the other, it took as
+  // long as a phase.  (The barrier words were written by earlier launches; no CTA gets past the first
+  // grid barrier before every CTA has read them.)
+  const size_t wi = (size_t)cta * FAST_WARPS + warp;
+  const uint32_t failed = __ldcg(P.epoch_base + 1), epoch_base = __ldcg(P.epoch_base);
+  const uint32_t ks_base = KSPLIT ? __ldcg(P.attn_cnt + cta % P.m.o_split) : 0u;
+  const uint64_t stream_off = P.m.stream_off[wi];
+  const int n_layer_chunks = P.m.chunk_cnt[wi * 2], n_head_chunks = P.m.chunk_cnt[wi * 2 + 1];
+  const int first_layer = P.layer_map ? P.layer_map[0] : 0;
 
   // per-CTA tables: tile lists, chunk sizes, rows of this forward
-  const size_t wi = (size_t)cta * FAST_WARPS + warp;
   if (tid < FOP_COUNT) M.ucnt[tid] = P.m.unit_cnt[cta * FOP_COUNT + tid];
   for (int i = tid; i < FOP_COUNT * FAST_MAX_UNITS; i += FAST_THREADS) {
     const int op = i / FAST_MAX_UNITS, u = i % FAST_MAX_UNITS;
-    const int cnt = P.m.unit_cnt[cta * FOP_COUNT + op];
-    M.utile[op][u] = u < cnt ? P.m.unit_tile[P.m.unit_off[cta * FOP_COUNT + op] + u] : 0;
+    const int cnt = P.m.unit_cnt[cta * FOP_COUNT + op], off = P.m.unit_off[cta * FOP_COUNT + op];
+    M.utile[op][u] = u < cnt ? P.m.unit_tile[off + u] : 0;
   }
   for (int i = lane; i < FAST_MAX_CHUNKS / 4; i += 32)
     reinterpret_cast<uint32_t*>(M.chunks[warp])[i] =
@@ -1199,8 +1202,8 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) fast_forward_kernel(const __g
   ring.ring = smem_u32(smem) + warp * P.ring_warp_bytes;
   ring.bars = smem_u32(&M.bars[warp][0]);
   ring.tab = M.chunks[warp];
-  ring.ncl = (uint32_t)P.m.chunk_cnt[wi * 2];
-  ring.nend = ring.ncl + (P.logits ? (uint32_t)P.m.chunk_cnt[wi * 2 + 1] : 0u);
+  ring.ncl = (uint32_t)n_layer_chunks;
+  ring.nend = ring.ncl + (P.logits ? (uint32_t)n_head_chunks : 0u);
   ring.layers_left = ring.ncl ? (uint32_t)P.L : 0u;
   ring.pc = 0;
   ring.slot = ring.parity = 0;
@@ -1217,9 +1220,9 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) fast_forward_kernel(const __g
   __syncwarp();  // also orders this warp's chunk table before its first use
   {
     uint32_t lb = 0;
-    for (uint32_t i = 0; i < ring.ncl; ++i) lb += ring.tab[i];
-    lb *= FAST_TILE_BYTES;
-    const uint8_t* base = P.m.wstream + P.m.stream_off[wi];
+    for (uint32_t i = lane; i < ring.ncl; i += 32) lb += ring.tab[i];
+    lb = __reduce_add_sync(0xffffffffu, lb) * FAST_TILE_BYTES;
+    const uint8_t* base = P.m.wstream + stream_off;
     if (lane == 0) {
       RingSide* sd = reinterpret_cast<RingSide*>(M.chunks[warp] + FAST_MAX_CHUNKS);
       sd->base = base;
@@ -1231,13 +1234,14 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) fast_forward_kernel(const __g
     __syncwarp();
     ring.mapped = P.layer_map != nullptr;
     ring.src = base;
-    if (ring.mapped) ring.src = base + (size_t)(ring.ncl ? P.layer_map[0] : P.n_src_layers) * lb;
+    if (ring.mapped) ring.src = base + (size_t)(ring.ncl ? first_layer : P.n_src_layers) * lb;
+  }
+  // a launch that failed earlier leaves the barrier words unusable: refuse to run on them
+  if (failed != 0u) {
+    if (cta == 0 && tid == 0) atomicOr(P.status, SSD_STATUS_TIMEOUT);
+    return;
   }
   for (int s = 0; s < P.nslot; ++s) ring_request(ring, (uint32_t)s, lane);
-  const uint32_t epoch_base = ld_acquire_u32(P.epoch_base);
-  // key-split variant: the slice counters are quiet between launches, and no CTA gets past the
-  // first grid barrier before every CTA has read its slice's value here
-  const uint32_t ks_base = KSPLIT ? ld_acquire_u32(P.attn_cnt + cta % P.m.o_split) : 0u;
   uint32_t epoch = 0;
   __syncthreads();
   trace_mark<TRACE>(P, n_trace);

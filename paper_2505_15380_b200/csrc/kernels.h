@@ -26,6 +26,8 @@ void launch_prefill_advance(const PrefillSegs& segs, const int32_t* ids, int32_t
 void launch_advance_len(int32_t* len, int32_t* pending, int b, int add, const int32_t* ids,
                         int pending_index, cudaStream_t st);
 
+// `n` words from pinned host memory.
+void launch_fetch_words(const uint32_t* host, uint32_t* dst, int n, cudaStream_t st);
 void launch_kv_restore(int32_t* len, int32_t* pending, const int32_t* src_len,
                        const int32_t* src_pending, int B, int cap, cudaStream_t st);
 void launch_advance_all(int32_t* len, int B, int add, int cap, int32_t* status, cudaStream_t st);
@@ -83,8 +85,8 @@ void launch_loop_finish(int32_t* draft_len, int32_t* draft_pending, int cap, int
                         const int32_t* next_token, int B, int32_t* out_tokens, int out_capacity,
                         int32_t* out_count, int32_t* accept_log, int n_rows, int32_t* iteration,
                         int32_t* recent_tokens, int ras_window, int32_t* status, cudaStream_t st);
-void launch_kv_commit(int32_t* len, int32_t* pending, const int32_t* accepted_len,
-                      const int32_t* next_token, int B, int cap, int max_gamma, int32_t* status,
-                      cudaStream_t st);
+// host_out (may be null): pinned host memory that gets [accepted_len | next_token] too.
+void launch_kv_commit(int32_t* len, int32_t* pending, const int32_t* accepted_len, const int32_t* next_token, int B, int cap,
+                      int max_gamma, int32_t* status, cudaStream_t st, int32_t* host_out = nullptr);
 
 }  // namespace ssd

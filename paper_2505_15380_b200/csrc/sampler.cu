@@ -763,11 +763,15 @@ cudaError_t launch_draft_sampler(const float* logits, int ld_logits, int V, cons
 // "Append to T_in" (Algorithm 1): the prefix grows by the k accepted tokens plus the new one.
 __global__ void kv_commit_kernel(int32_t* len, int32_t* pending, const int32_t* accepted_len,
                                  const int32_t* next_token, int B, int cap, int max_gamma,
-                                 int32_t* status) {
+                                 int32_t* status, int32_t* host_out) {
   tc_pdl_enter();
   int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
-  const int k = accepted_len[b];
+  const int k = accepted_len[b], y = next_token[b];
+  if (host_out) {
+    host_out[b] = k;
+    host_out[B + b] = y;
+  }
   if (k < 0 || k > max_gamma) {  // not an accepted length: the stream stays as it is
     atomicOr(status, SSD_STATUS_BAD_TOKEN);
     return;
@@ -778,14 +782,13 @@ __global__ void kv_commit_kernel(int32_t* len, int32_t* pending, const int32_t* 
     nl = cap;
   }
   len[b] = nl;
-  pending[b] = next_token[b];
+  pending[b] = y;
 }
 
-void launch_kv_commit(int32_t* len, int32_t* pending, const int32_t* accepted_len,
-                      const int32_t* next_token, int B, int cap, int max_gamma, int32_t* status,
-                      cudaStream_t st) {
+void launch_kv_commit(int32_t* len, int32_t* pending, const int32_t* accepted_len, const int32_t* next_token, int B, int cap,
+                      int max_gamma, int32_t* status, cudaStream_t st, int32_t* host_out) {
   tc_launch_pdl(kv_commit_kernel, dim3((B + 127) / 128), dim3(128), 0, st, len, pending, accepted_len, next_token, B,
-                cap, max_gamma, status);
+                cap, max_gamma, status, host_out);
   count_launch();
 }
 

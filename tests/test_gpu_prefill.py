@@ -52,3 +52,24 @@ def test_verify_after_a_prefill_of_several_chunks():
     shape = synth.ModelShape(2, 128, 4, 2, 64, 256, 300, 8, 1e4, weight_dtype=synth.BF16)
     wl = synth.Workload("prefill", shape, shape, 4, 4, 0.8, 25, (1300, 17, 900, 260), 2, 5, 6)
     run_case(wl, beta=0.4, sigma=1.0, logit_tol=2e-3)
+
+
+def test_short_prompts_beside_others_equal_prompts_alone():
+    """Prompts of at most 16 rows take the persistent kernel, whoever joins beside them."""
+    from paper_2505_15380_b200 import binding
+    lens = [300, 17, 2, 40, 9]
+    shape = synth.ModelShape(3, 128, 4, 2, 64, 256, 301, 8, 1e4, weight_dtype=synth.BF16)
+    wl = synth.Workload("prefill", shape, shape, len(lens), 3, 1.0, 0, tuple(lens), 2, 5, 6)
+    model = binding.Model(shape, synth.weights_blob(shape, synth.make_weights(shape, 5)))
+    prefixes = [synth.make_prefix(wl, b) for b in range(len(lens))]
+    together, alone = (binding.Streams(model, len(lens), max(lens) + 8, 3) for _ in range(2))
+    together.kv.zero_()
+    alone.kv.zero_()
+    together.prefill(prefixes)
+    for b in range(len(lens)):
+        alone.prefill([p if i == b else np.zeros(0, np.int32) for i, p in enumerate(prefixes)])
+    for gs in (together, alone):
+        assert gs.last_status() == 0
+        n, pend = gs.get_state()
+        assert list(n) == [x - 1 for x in lens] and list(pend) == [int(p[-1]) for p in prefixes]
+    assert torch.equal(together.kv, alone.kv)
