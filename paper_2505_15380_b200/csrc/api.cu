@@ -685,10 +685,9 @@ int draft_step_impl(ssd_model* draft, ssd_streams* ds, const int32_t* ids, int n
     rc = forward(draft, ds, rm, nullptr, ds->logits, st);
   }
   if (rc != SSD_OK) return rc;
-  launch_advance_all(ds->len, ds->B, n_in, ds->cap, ds->status, st);
   SSD_CUDA(launch_draft_sampler(ds->logits + (size_t)(n_in - 1) * V, n_in * V, V, uniform, ds->B,
                                 1.0f / params->temperature, params->top_k, params->top_p, out_token, tok_stride, out_prob,
-                                prob_stride, ds->pending, ds->status, st));
+                                prob_stride, ds->pending, ds->len, n_in, ds->cap, ds->status, st));
   return SSD_OK;
 }
 
@@ -1294,13 +1293,12 @@ int ssd_iteration(ssd_model* target, ssd_streams* ts, ssd_model* draft, ssd_stre
   rc = ssd_verify(target, ts, io->dev_draft_tokens, io->dev_draft_probs, ts->st_uni, params,
                   io->dev_accepted_len, io->dev_next_token, nullptr, stream);  // Eq. 4-6
   if (rc != SSD_OK) return rc;
-  rc = ssd_kv_commit(ts, io->dev_accepted_len, io->dev_next_token, stream);
-  if (rc != SSD_OK) return rc;
-  launch_loop_finish(ds->len, ds->pending, ds->cap, io->dev_in_ids, io->dev_draft_tokens, gamma,
+  launch_loop_finish(ts->len, ts->pending, ts->cap, ds->len, ds->pending, ds->cap, io->dev_in_ids, io->dev_draft_tokens, gamma,
                      io->dev_accepted_len, io->dev_next_token, B, io->dev_out_tokens, io->out_capacity,
                      io->dev_out_count, io->dev_accept_log, io->n_iterations, io->dev_iteration,
                      params->ras_window > 0 ? const_cast<int32_t*>(params->dev_recent_tokens) : nullptr,
                      params->ras_window, ts->status, st);
+  release_pages(ts, st);
   release_pages(ds, st);
   SSD_CUDA(cudaGetLastError());
   return SSD_OK;

@@ -171,22 +171,4 @@ void launch_kv_restore(int32_t* len, int32_t* pending, const int32_t* src_len,
   count_launch();
 }
 
-// Draft bookkeeping: every stream's committed length grows by `add`.
-__global__ void advance_all_kernel(int32_t* len, int B, int add, int cap, int32_t* status) {
-  tc_pdl_enter();
-  int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= B) return;
-  int nl = len[b] + add;
-  if (nl > cap) {
-    atomicOr(status, SSD_STATUS_KV_OVERFLOW);
-    nl = cap;
-  }
-  len[b] = nl;
-}
-
-void launch_advance_all(int32_t* len, int B, int add, int cap, int32_t* status, cudaStream_t st) {
-  tc_launch_pdl(advance_all_kernel, dim3((B + 127) / 128), dim3(128), 0, st, len, B, add, cap, status);
-  count_launch();
-}
-
 }  // namespace ssd

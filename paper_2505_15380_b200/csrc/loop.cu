@@ -32,6 +32,7 @@ void launch_loop_stage_uniforms(const float* pool, int n_rows, const int32_t* it
 }
 
 // End of an iteration, per stream: the prefix grew by x_1..x_k and the new token y.
+//  * target cache: committed (len += 1 + k, y pending);
 //  * emitted tokens: x_1..x_k, y are appended to the stream's output (as far as it has room);
 //  * draft cache: the gamma draft steps left K/V for the old pending token and x_1..x_{gamma-1}.
 //    The next iteration's first draft step always feeds two ids, [token before y, y], at the
@@ -39,7 +40,7 @@ void launch_loop_stage_uniforms(const float* pool, int n_rows, const int32_t* it
 //    K/V of x_gamma; otherwise it recomputes one cached row with the same inputs.  One rule for
 //    every stream, so a batch needs no host decision;
 //  * in_ids[b] = [k > 0 ? x_k : the token that was pending, y].
-__global__ void loop_finish_kernel(int32_t* draft_len, int32_t* draft_pending, int cap, int32_t* in_ids,
+__global__ void loop_finish_kernel(int32_t* target_len, int32_t* target_pending, int target_cap, int32_t* draft_len, int32_t* draft_pending, int cap, int32_t* in_ids,
                                    const int32_t* __restrict__ draft_tokens, int gamma,
                                    const int32_t* __restrict__ accepted_len,
                                    const int32_t* __restrict__ next_token, int B, int32_t* out_tokens,
@@ -56,6 +57,10 @@ __global__ void loop_finish_kernel(int32_t* draft_len, int32_t* draft_pending, i
     if (accept_log) accept_log[(size_t)it * B + b] = k;
     if (k >= 0) {
       const int y = next_token[b];
+      const int tl = max(target_len[b], 0) + 1 + k;
+      if (tl > target_cap) atomicOr(status, SSD_STATUS_KV_OVERFLOW);
+      target_len[b] = min(tl, target_cap);
+      target_pending[b] = y;
       int n = out_count[b];
       for (int i = 0; i <= k; ++i) {
         if (n < out_capacity) out_tokens[(size_t)b * out_capacity + n] = i < k ? draft_tokens[b * gamma + i] : y;
@@ -81,13 +86,13 @@ __global__ void loop_finish_kernel(int32_t* draft_len, int32_t* draft_pending, i
   if (threadIdx.x == 0) *iteration = *iteration + 1;
 }
 
-void launch_loop_finish(int32_t* draft_len, int32_t* draft_pending, int cap, int32_t* in_ids,
+void launch_loop_finish(int32_t* target_len, int32_t* target_pending, int target_cap, int32_t* draft_len, int32_t* draft_pending, int cap, int32_t* in_ids,
                         const int32_t* draft_tokens, int gamma, const int32_t* accepted_len,
                         const int32_t* next_token, int B, int32_t* out_tokens, int out_capacity,
                         int32_t* out_count, int32_t* accept_log, int n_rows, int32_t* iteration,
                         int32_t* recent_tokens, int ras_window, int32_t* status, cudaStream_t st) {
   // one block: every thread reads the iteration counter before the last thread advances it
-  tc_launch_pdl(loop_finish_kernel, dim3(1), dim3(1024), 0, st, draft_len, draft_pending, cap, in_ids, draft_tokens,
+  tc_launch_pdl(loop_finish_kernel, dim3(1), dim3(1024), 0, st, target_len, target_pending, target_cap, draft_len, draft_pending, cap, in_ids, draft_tokens,
                 gamma, accepted_len, next_token, B, out_tokens, out_capacity, out_count, accept_log, n_rows,
                 iteration, recent_tokens, ras_window, status);
   count_launch();

@@ -15,6 +15,7 @@
 
 #include "kernels.h"
 #include "tc.h"
+#include "tc_ptx.cuh"
 
 namespace ssd {
 
@@ -601,6 +602,29 @@ __device__ __forceinline__ float q_value(float v, int t, const RowStats& st, int
   return q;
 }
 
+// A row's token and flag; the last row of a stream to arrive finds the first rejection and that row's token.
+// One warp; lane 0's y and flag count.
+__device__ __forceinline__ void finish_row(int y, bool flag, int b, int r, int R, int32_t* row_words, int32_t* counters,
+                                           int32_t* accepted_len, int32_t* next_token) {
+  const int lane = threadIdx.x & 31;
+  int prev = 0;
+  if (lane == 0) {
+    row_words[b * R + r] = y * 2 + (int)flag;
+    __threadfence();
+    prev = atomicAdd(&counters[b], 1);
+  }
+  if (__shfl_sync(0xffffffffu, prev, 0) != R - 1) return;
+  __threadfence();
+  const int w = lane < R ? __ldcg(&row_words[b * R + lane]) : 1;  // R is at most 16
+  const uint32_t rejected = __ballot_sync(0xffffffffu, lane < R - 1 && !(w & 1));
+  const int k = rejected ? __ffs(rejected) - 1 : R - 1;
+  if (lane == k) {
+    counters[b] = 0;
+    accepted_len[b] = k;
+    next_token[b] = w >> 1;
+  }
+}
+
 // Grid (R, B), R = gamma + 1.
 __global__ void __launch_bounds__(SAMP_THREADS)
 verify_sampler_kernel(const float* __restrict__ logits, int V,
@@ -662,24 +686,255 @@ verify_sampler_kernel(const float* __restrict__ logits, int V,
     y = block_inverse_cdf(z, V, u.y, sm, &total);
     if (y < 0) y = 0;
   }
-  // ---- the last CTA of this stream: first rejection, and that row's token ----
-  if (tid >= 32) return;
-  int prev = 0;
+  if (tid < 32) finish_row(y, flag, b, r, R, row_words, counters, accepted_len, next_token);
+}
+
+// ---- plain rows (softmax over the whole vocabulary: no cut, no repetition window), split over a cluster
+//
+// One CTA per row is bound by that SM's instructions (6564 ids take 18 thousand cycles in all) while the
+// rest of the chip is idle.  Eight CTAs take an eighth each and exchange three numbers - largest value, sum,
+// mass of the draw - as remote stores that complete on the receivers' barriers; a cluster barrier with
+// its fence would cost a thousand cycles each time.  Every CTA adds the contributions in rank order.
+constexpr int PL_CLUSTER = 8, PL_THREADS = 256, PL_WARPS = PL_THREADS / 32;
+enum { PL_MAX, PL_SUM, PL_MASS, PL_FLAG, PL_MASS2, PL_SLOTS };
+
+struct PlainSmem {
+  double slot[PL_SLOTS][PL_CLUSTER];  // what the CTAs of the cluster sent
+  unsigned long long bar[3 + 1];      // of max; sum; mass and flag; mass of the second draw
+  double red[PL_WARPS];
+  double scan[PL_THREADS];
+  float red_f[PL_WARPS];
+  int y, abort;
+};
+
+__device__ __forceinline__ void plain_send(PlainSmem& sm, int what, int bar, double v) {  // lanes 0 .. PL_CLUSTER - 1 of warp 0
+  const uint32_t to = threadIdx.x, me = tcx::cluster_rank();
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];"
+               ::"r"(tcx::map_rank(tcx::smem_u32(&sm.slot[what][me]), to)), "l"(__double_as_longlong(v)),
+                 "r"(tcx::map_rank(tcx::smem_u32(&sm.bar[bar]), to))
+               : "memory");
+}
+// Sum over the CTA, valid in warp 0.
+__device__ __forceinline__ double plain_block_sum(double v, PlainSmem& sm) {
+  v = warp_sum_d(v);
+  if ((threadIdx.x & 31) == 0) sm.red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  return warp_sum_d(threadIdx.x < PL_WARPS ? sm.red[threadIdx.x] : 0.0);
+}
+
+// The draw over the weights w[0..n) of the cluster's CTAs: each CTA's running sums, the masses exchanged, and the
+// CTA in which u * total falls finds the id.  Returns its place in this CTA's slice, -1 in the other CTAs, -2
+// in all of them where there is no mass.
+__device__ int plain_draw(const float* w, int n, float u, int what, int bar, double flag, PlainSmem& sm) {
+  const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5, me = (int)tcx::cluster_rank();
+  const int seg = (n + PL_THREADS - 1) / PL_THREADS, i0 = min(tid * seg, n), i1 = min(i0 + seg, n);
+  double s = 0.0;
+  for (int i = i0; i < i1; ++i) s += (double)w[i];
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const double v = __shfl_up_sync(0xffffffffu, s, o);
+    if (lane >= o) s += v;
+  }
+  if (lane == 31) sm.red[wp] = s;
+  if (tid == 0) sm.y = -1;
+  __syncthreads();
+  double ahead = 0.0, mass = 0.0;
+#pragma unroll
+  for (int i = 0; i < PL_WARPS; ++i) {
+    if (i == wp) ahead = mass;
+    mass += sm.red[i];
+  }
+  if (tid < PL_CLUSTER) {
+    plain_send(sm, what, bar, mass);
+    if (what == PL_MASS) plain_send(sm, PL_FLAG, bar, flag);
+  }
+  sm.scan[tid] = ahead + s;
+  __syncthreads();
+  tcx::mbar_wait(tcx::smem_u32(&sm.bar[bar]), 0u, &sm.abort);
+  double total = 0.0, before = 0.0;
+  int last = -1;  // last CTA with mass
+  for (int i = 0; i < PL_CLUSTER; ++i) {
+    if (i == me) before = total;
+    if (sm.slot[what][i] > 0.0) last = i;
+    total += sm.slot[what][i];
+  }
+  if (!(total > 0.0)) return -2;
+  const double target = (double)u * total;
+  int owner = -1;
+  double run = 0.0;
+  for (int i = 0; i < PL_CLUSTER; ++i) {
+    run += sm.slot[what][i];
+    if (owner < 0 && target < run) owner = i;
+  }
+  if (me != (owner < 0 ? last : owner)) return -1;
+  const double excl = before + (tid == 0 ? 0.0 : sm.scan[tid - 1]), incl = before + sm.scan[tid];
+  if (owner >= 0 && excl <= target && target < incl) {
+    double r = excl;
+    int y = -1;
+    for (int i = i0; i < i1; ++i) {
+      r += (double)w[i];
+      if (w[i] > 0.f) {
+        y = i;
+        if (r > target) break;
+      }
+    }
+    sm.y = y;
+  }
+  __syncthreads();
+  if (sm.y < 0 && tid == 0) {  // u * total rounded up to this CTA's end: its last id with mass
+    int i = n - 1;
+    while (i > 0 && !(w[i] > 0.f)) --i;
+    sm.y = i;
+  }
+  __syncthreads();
+  return sm.y;
+}
+
+struct PlainArgs {
+  const float* logits;
+  size_t ld;  // from one row's logits to the next one's
+  int V, R;   // rows per stream (drafting: 1)
+  float inv_t;
+  const float* uniforms;  // verify: [B, R, 2]; drafting: [B]
+  // verify
+  const int32_t* draft_tokens;
+  const float* draft_probs;
+  float beta;
+  int32_t *row_words, *counters, *accepted_len, *next_token;
+  // drafting
+  int32_t* out_token;
+  int tok_stride;
+  float* out_prob;
+  size_t prob_stride;
+  int32_t *pending, *len;
+  int add, cap;
+  int32_t* status;
+};
+
+// Grid (R * PL_CLUSTER, B), clusters along x.
+template <bool DRAFT>
+__global__ void __launch_bounds__(PL_THREADS) plain_sampler_kernel(const __grid_constant__ PlainArgs A) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  PlainSmem& sm = *reinterpret_cast<PlainSmem*>(smem_raw);
+  float* z = reinterpret_cast<float*>(smem_raw + sizeof(PlainSmem));
+  const int tid = threadIdx.x, lane = tid & 31, me = (int)tcx::cluster_rank();
+  const int r = blockIdx.x / PL_CLUSTER, b = blockIdx.y, R = A.R, gamma = R - 1, V = A.V;
+  const int per = (V + PL_CLUSTER - 1) / PL_CLUSTER, t0 = min(me * per, V), n = min(per, V - t0);
+  const float* prow = !DRAFT && r < gamma ? A.draft_probs + ((size_t)b * gamma + r) * V : nullptr;
   if (tid == 0) {
-    row_words[b * R + r] = y * 2 + flag;
-    __threadfence();
-    prev = atomicAdd(&counters[b], 1);
+    for (int i = 0; i < 4; ++i) tcx::mbar_init(tcx::smem_u32(&sm.bar[i]), 1);
+    sm.abort = 0;
+    tcx::mbar_init_fence();
+    for (int i = 0; i < 4; ++i) tcx::mbar_expect_tx(tcx::smem_u32(&sm.bar[i]), (i == 2 ? 16u : 8u) * PL_CLUSTER);
   }
-  if (__shfl_sync(0xffffffffu, prev, 0) != R - 1) return;
-  __threadfence();
-  const int w = tid < R ? __ldcg(&row_words[b * R + tid]) : 1;  // R is at most 16
-  const uint32_t rejected = __ballot_sync(0xffffffffu, tid < gamma && !(w & 1));
-  const int k = rejected ? __ffs(rejected) - 1 : gamma;
-  if (tid == k) {
-    counters[b] = 0;
-    accepted_len[b] = k;
-    next_token[b] = w >> 1;
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  if (prow)  // (a hint: whoever writes the row may still be at it)
+    for (int i = tid * 32; i < n; i += PL_THREADS * 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(prow + t0 + i));
+  tc_pdl_enter();
+  int x = -1;
+  if (!DRAFT && tid == 0 && prow) x = A.draft_tokens[b * gamma + r];
+  const float u = DRAFT ? A.uniforms[b] : A.uniforms[((size_t)b * R + r) * 2 + 1];
+  const float ur = DRAFT ? 0.f : A.uniforms[((size_t)b * R + r) * 2];
+  const float* lrow = A.logits + (size_t)(b * R + r) * A.ld + t0;
+  float mx = -CUDART_INF_F;
+  int bad = 0;
+#pragma unroll 4
+  for (int i = tid; i < n; i += PL_THREADS) {
+    const float v = lrow[i];
+    if (!isfinite(v)) bad = 1;
+    z[i] = v * A.inv_t;
+    mx = fmaxf(mx, z[i]);
   }
+  float px = 0.f;
+  if (!DRAFT && prow && x >= t0 && x < t0 + n) px = prow[x];
+  mx = warp_max(mx);
+  if (lane == 0) sm.red_f[tid >> 5] = mx;
+  bad = __syncthreads_or(bad);
+  if (bad && tid == 0) atomicOr(A.status, SSD_STATUS_NONFINITE);
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // the other CTAs' barriers exist
+  if (tid < 32) {
+    mx = warp_max(lane < PL_WARPS ? sm.red_f[lane] : -CUDART_INF_F);
+    if (lane < PL_CLUSTER) plain_send(sm, PL_MAX, 0, (double)mx);
+  }
+  tcx::mbar_wait(tcx::smem_u32(&sm.bar[0]), 0u, &sm.abort);
+  float zmax = (float)sm.slot[PL_MAX][0];
+#pragma unroll
+  for (int i = 1; i < PL_CLUSTER; ++i) zmax = fmaxf(zmax, (float)sm.slot[PL_MAX][i]);
+  double s = 0.0;
+#pragma unroll 2
+  for (int i = tid; i < n; i += PL_THREADS) {
+    const float e = expf(z[i] - zmax);
+    z[i] = e;
+    s += (double)e;
+  }
+  s = plain_block_sum(s, sm);
+  if (tid < PL_CLUSTER) plain_send(sm, PL_SUM, 1, s);
+  tcx::mbar_wait(tcx::smem_u32(&sm.bar[1]), 0u, &sm.abort);
+  s = 0.0;
+#pragma unroll
+  for (int i = 0; i < PL_CLUSTER; ++i) s += sm.slot[PL_SUM][i];
+  const float sum = (float)s;
+  int flag = 0;
+  if (!DRAFT && prow && tid == 0) {  // Eq. 5: accept x_i iff r_i < min(1, q_i(x_i) / p_i(x_i)) + beta
+    // a draft token or probability that cannot be one is rejected, never accepted
+    if (x < 0 || x >= V) {
+      if (me == 0) atomicOr(A.status, SSD_STATUS_BAD_TOKEN);
+    } else if (x >= t0 && x < t0 + n) {
+      if (!(px >= 0.f) || !isfinite(px)) {
+        atomicOr(A.status, SSD_STATUS_BAD_PROB);
+      } else {
+        const float qx = z[x - t0] / sum, ratio = px <= qx ? 1.f : qx / px;
+        flag = ur < ratio + A.beta;
+      }
+    }
+  }
+  flag = __syncthreads_or(flag);  // and the value above is read: z becomes the weights of the draw
+#pragma unroll 4
+  for (int i = tid; i < n; i += PL_THREADS) {
+    const float q = z[i] / sum;
+    if (DRAFT) A.out_prob[(size_t)b * A.prob_stride + t0 + i] = q;
+    z[i] = prow ? fmaxf(0.f, q - prow[t0 + i]) : q;
+  }
+  __syncthreads();
+  int y = plain_draw(z, n, u, PL_MASS, 2, (double)flag, sm);
+  if (!DRAFT && y == -2) {  // residual has no mass (numerical corner): draw from q_r itself
+    __syncthreads();
+    for (int i = tid; i < n; i += PL_THREADS) z[i] = expf(lrow[i] * A.inv_t - zmax) / sum;
+    __syncthreads();
+    y = plain_draw(z, n, u, PL_MASS2, 3, 0.0, sm);
+  }
+  if (y == -2 && me == 0) y = 0;
+  if (tid == 0 && sm.abort) atomicOr(A.status, SSD_STATUS_TIMEOUT);
+  if (y < 0 || tid >= 32) return;
+  y += t0;
+  if (DRAFT) {
+    if (tid == 0) {
+      A.out_token[(size_t)b * A.tok_stride] = y;
+      A.pending[b] = y;
+      const int nl = A.len[b] + A.add;  // the rows of the forward are committed
+      if (nl > A.cap) atomicOr(A.status, SSD_STATUS_KV_OVERFLOW);
+      A.len[b] = min(nl, A.cap);
+    }
+    return;
+  }
+  double f = 0.0;
+  for (int i = 0; i < PL_CLUSTER; ++i) f += sm.slot[PL_FLAG][i];
+  finish_row(y, f > 0.0, b, r, R, A.row_words, A.counters, A.accepted_len, A.next_token);
+}
+
+// Plain rows take the cluster kernel while its CTAs leave most of an SM to each other: 5 rows 14.3 -> 11.7 us,
+// 24 rows 14.4 -> 12.3, 96 rows the same.
+bool plain_rows(int rows, int V, int top_k, float top_p, int ras_window) {
+  return !(top_k > 0 && top_k < V) && !(top_p > 0.f && top_p < 1.f) && ras_window <= 0 && rows <= 64;
+}
+template <bool DRAFT>
+cudaError_t launch_plain(const PlainArgs& a, int B, cudaStream_t st) {
+  const size_t smem = sizeof(PlainSmem) + (size_t)((a.V + PL_CLUSTER - 1) / PL_CLUSTER) * sizeof(float);
+  const cudaError_t e = tc_launch_pdl_cluster(plain_sampler_kernel<DRAFT>, dim3(a.R * PL_CLUSTER, B), dim3(PL_THREADS),
+                                              PL_CLUSTER, smem, st, a);
+  if (e != cudaSuccess) return e;
+  count_launch();
+  return cudaGetLastError();
 }
 
 cudaError_t launch_verify_sampler(const float* logits, int V, const int32_t* draft_tokens,
@@ -693,6 +948,24 @@ cudaError_t launch_verify_sampler(const float* logits, int V, const int32_t* dra
   if (ras_window > 0) {
     if (ras_window > RAS_MAX_WIN || !recent_tokens) return cudaErrorInvalidValue;
     ras = Ras{ras_window, (float)ras_window * ras_tau, recent_tokens};
+  }
+  if (plain_rows(B * (gamma + 1), V, top_k, top_p, ras_window)) {
+    PlainArgs a{};
+    a.logits = logits;
+    a.ld = (size_t)V;
+    a.V = V;
+    a.R = gamma + 1;
+    a.inv_t = inv_temperature;
+    a.uniforms = uniforms;
+    a.draft_tokens = draft_tokens;
+    a.draft_probs = draft_probs;
+    a.beta = beta;
+    a.row_words = row_words;
+    a.counters = counters;
+    a.accepted_len = accepted_len;
+    a.next_token = next_token;
+    a.status = status;
+    return launch_plain<false>(a, B, st);
   }
   size_t smem = sizeof(SampSmem) + (size_t)V * sizeof(float);
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
@@ -715,7 +988,7 @@ __global__ void __launch_bounds__(SAMP_THREADS)
 draft_sampler_kernel(const float* __restrict__ logits, int ld_logits, int V,
                      const float* __restrict__ uniform, float inv_t, int top_k, float top_p,
                      int32_t* __restrict__ out_token, int tok_stride, float* __restrict__ out_prob,
-                     size_t prob_stride, int32_t* pending, int32_t* status) {
+                     size_t prob_stride, int32_t* pending, int32_t* len, int add, int cap, int32_t* status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SampSmem& sm = *reinterpret_cast<SampSmem*>(smem_raw);
   float* z = reinterpret_cast<float*>(smem_raw + sizeof(SampSmem));
@@ -739,14 +1012,36 @@ draft_sampler_kernel(const float* __restrict__ logits, int ld_logits, int V,
   if (threadIdx.x == 0) {
     out_token[(size_t)b * tok_stride] = y;
     pending[b] = y;
+    const int nl = len[b] + add;  // the rows of the forward are committed
+    if (nl > cap) atomicOr(status, SSD_STATUS_KV_OVERFLOW);
+    len[b] = min(nl, cap);
   }
 }
 
 cudaError_t launch_draft_sampler(const float* logits, int ld_logits, int V, const float* uniform,
                                  int B, float inv_temperature, int top_k, float top_p,
                                  int32_t* out_token, int tok_stride, float* out_prob_row,
-                                 size_t prob_stride, int32_t* pending, int32_t* status,
-                                 cudaStream_t st) {
+                                 size_t prob_stride, int32_t* pending, int32_t* len, int add, int cap,
+                                 int32_t* status, cudaStream_t st) {
+  if (plain_rows(B, V, top_k, top_p, 0)) {
+    PlainArgs a{};
+    a.logits = logits;
+    a.ld = (size_t)ld_logits;
+    a.V = V;
+    a.R = 1;
+    a.inv_t = inv_temperature;
+    a.uniforms = uniform;
+    a.out_token = out_token;
+    a.tok_stride = tok_stride;
+    a.out_prob = out_prob_row;
+    a.prob_stride = prob_stride;
+    a.pending = pending;
+    a.len = len;
+    a.add = add;
+    a.cap = cap;
+    a.status = status;
+    return launch_plain<true>(a, B, st);
+  }
   size_t smem = sizeof(SampSmem) + (size_t)V * sizeof(float);
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
   if (smem > 48 * 1024) {
@@ -755,7 +1050,8 @@ cudaError_t launch_draft_sampler(const float* logits, int ld_logits, int V, cons
     if (e != cudaSuccess) return e;
   }
   tc_launch_pdl(draft_sampler_kernel, dim3(B), dim3(SAMP_THREADS), smem, st, logits, ld_logits, V, uniform,
-                inv_temperature, top_k, top_p, out_token, tok_stride, out_prob_row, prob_stride, pending, status);
+                inv_temperature, top_k, top_p, out_token, tok_stride, out_prob_row, prob_stride, pending, len, add,
+                cap, status);
   count_launch();
   return cudaGetLastError();
 }

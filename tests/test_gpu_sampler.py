@@ -55,3 +55,33 @@ def test_cuts(V, kind):
                 assert int(y[b]) == o["y"]
                 compared += 1
     assert compared >= 8
+
+
+@pytest.mark.parametrize("B", [1, 19, 40])
+@pytest.mark.parametrize("V", [2, 7, 1025, 2047, 6564, 46080])
+def test_plain_rows(V, B):
+    """Softmax over the whole vocabulary, on both sides of the number of rows up to which a cluster takes a row."""
+    from paper_2505_15380_b200 import binding
+    dev = torch.device("cuda:0")
+    rng = np.random.default_rng(V + B)
+    gamma = 4
+    lg = _rows("normal", B * (gamma + 1), V, rng).reshape(B, gamma + 1, V)
+    p = synth.random_prob_rows(B * gamma, V, seed=V, sharpness=1.0).reshape(B, gamma, V)
+    x = synth.sample_from_rows(p.reshape(-1, V), seed=V + 1).reshape(B, gamma).astype(np.int32)
+    u = synth.verify_uniforms(V, B, gamma + 1)
+    k, y = (torch.full((B,), -2, dtype=torch.int32, device=dev) for _ in range(2))
+    compared = 0
+    for beta in (0.0, 0.4):
+        t = [torch.from_numpy(a).to(dev).contiguous() for a in (lg, x, p, u)]
+        binding.accept_noalloc(*t, binding.VerifyParams(gamma, 1.0, 0, beta), k, y)
+        torch.cuda.synchronize()
+        for b in range(B):
+            q = np.stack([orc.transform(r.astype(np.float64), 1.0, 0) for r in lg[b]])
+            o = orc.accept_step(q, p[b], x[b], u[b], beta)
+            if any(abs(a - float(u[b, i, 0])) < 1e-5 for i, a in enumerate(o["thresholds"])):
+                continue
+            assert int(k[b]) == o["k"]
+            if o["draw_margin"] >= 1e-5:
+                assert int(y[b]) == o["y"]
+                compared += 1
+    assert compared >= B
