@@ -18,10 +18,12 @@
 
 namespace ssd {
 
-constexpr int ATTN_WARPS = 4;
+// A warp per query row of the kv head, as far as that goes: a row is a chain of shuffles and sums, and three
+// rows one after the other took 12 us of a 68 us forward (4 warps; 10 rows).
+constexpr int ATTN_MIN_WARPS = 4, ATTN_MAX_WARPS = 16;
 
 template <typename T, int HD>
-__global__ void __launch_bounds__(ATTN_WARPS * 32)
+__global__ void __launch_bounds__(ATTN_MAX_WARPS * 32)
 attn_split_kernel(const float* __restrict__ qkv, const float* __restrict__ cs, T* __restrict__ kv_layer,
                   const int32_t* __restrict__ len, RowMap rm, int cap, int Hq, int Hkv, float scale,
                   float* __restrict__ part, int nsplit_max, int32_t* status) {
@@ -84,7 +86,7 @@ attn_split_kernel(const float* __restrict__ qkv, const float* __restrict__ cs, T
     Qs[row * HD + j + HD / 2] = (x2 * c.x + x1 * c.y) * scale;
   }
   __syncthreads();
-  for (int row = warp; row < NQ; row += ATTN_WARPS) {
+  for (int row = warp; row < NQ; row += (int)blockDim.x >> 5) {
     const int r = row / G, hl = row % G;
     const int last_visible = L + r;      // row r sees keys 0..len+r
     float m_run = -CUDART_INF_F, l_run = 0.f, acc[NI];
@@ -109,6 +111,7 @@ attn_split_kernel(const float* __restrict__ qkv, const float* __restrict__ cs, T
 #pragma unroll
       for (int i = 0; i < NI; ++i) acc[i] *= corr;
       const int lim = min(32, nk - t0);
+#pragma unroll 8
       for (int kk = 0; kk < lim; ++kk) {
         float pk = __shfl_sync(0xffffffffu, p, kk);
         const float* vr = Vs + (t0 + kk) * HD;
@@ -165,7 +168,8 @@ static cudaError_t launch_t(const float* qkv, const float* cs, void* kv_layer, c
     if (e != cudaSuccess) return e;
   }
   dim3 grid(nsplit_max, Hkv, rm.nb);
-  tc_launch_pdl(kern, grid, dim3(ATTN_WARPS * 32), smem, st, qkv, cs, (T*)kv_layer, len, rm, cap, Hq, Hkv,
+  const int warps = NQ < ATTN_MIN_WARPS ? ATTN_MIN_WARPS : NQ > ATTN_MAX_WARPS ? ATTN_MAX_WARPS : NQ;
+  tc_launch_pdl(kern, grid, dim3(warps * 32), smem, st, qkv, cs, (T*)kv_layer, len, rm, cap, Hq, Hkv,
                 1.0f / sqrtf((float)HD), part, nsplit_max, status);
   count_launch();
   return cudaGetLastError();
