@@ -78,7 +78,19 @@ gemm_simt_kernel(const SimtSrc S, const T* __restrict__ W,
   };
   const int c_first = lane + 32 * ks;
   if (active && c_first < kc_max >> 3) load_weights(0, c_first, kc_max >> 3);
+  // what the epilogue reads, requested now
+  const bool mine = active && ks == 0 && lane < GEMM_MT && m0 + lane < M;
+  const size_t at = (size_t)(m0 + lane) * ldc + n0;
+  float b0 = 0.f, b1 = 0.f, c0 = 0.f, c1 = 0.f;
+  if (EPI == EPI_STORE_F32 && mine && bias) {
+    b0 = to_f32<T>(bias[n0]);
+    b1 = has1 ? to_f32<T>(bias[n0 + 1]) : 0.f;
+  }
   tc_pdl_enter();
+  if (EPI == EPI_RESIDUAL && mine) {
+    c0 = C[at];
+    c1 = has1 ? C[at + 1] : 0.f;
+  }
   for (int k0 = 0; k0 < K; k0 += GEMM_KC) {
     const int kc = min(GEMM_KC, K - k0);  // multiple of 8
     __syncthreads();
@@ -142,48 +154,39 @@ gemm_simt_kernel(const SimtSrc S, const T* __restrict__ W,
       }
     }
   }
+  // lane r finishes row r (one lane after the other, the residual's loads and stores were a chain)
+  float v0 = 0.f, v1 = 0.f;
 #pragma unroll
   for (int r = 0; r < GEMM_MT; ++r) {
-    acc0[r] = warp_sum(acc0[r]);
-    acc1[r] = warp_sum(acc1[r]);
+    const float s0 = warp_sum(acc0[r]), s1 = warp_sum(acc1[r]);
+    if (lane == r) {
+      v0 = s0;
+      v1 = s1;
+    }
   }
   if (KS > 1) {
-    if (lane == 0) {
-#pragma unroll
-      for (int r = 0; r < GEMM_MT; ++r) {
-        red[warp][r][0] = acc0[r];
-        red[warp][r][1] = acc1[r];
-      }
+    if (lane < GEMM_MT) {
+      red[warp][lane][0] = v0;
+      red[warp][lane][1] = v1;
     }
     __syncthreads();
-    if (ks == 0 && lane == 0) {
-#pragma unroll
-      for (int r = 0; r < GEMM_MT; ++r) {
-        float s0 = 0.f, s1 = 0.f;
-        for (int j = 0; j < KS; ++j) {  // fixed order: bit-reproducible
-          s0 += red[warp + j][r][0];
-          s1 += red[warp + j][r][1];
-        }
-        acc0[r] = s0;
-        acc1[r] = s1;
+    if (ks == 0 && lane < GEMM_MT) {
+      v0 = v1 = 0.f;
+      for (int j = 0; j < KS; ++j) {  // fixed order: bit-reproducible
+        v0 += red[warp + j][lane][0];
+        v1 += red[warp + j][lane][1];
       }
     }
   }
-  if (!active || ks != 0 || lane != 0) return;
-#pragma unroll
-  for (int r = 0; r < GEMM_MT; ++r) {
-    int m = m0 + r;
-    if (m >= M) break;
-    if (EPI == EPI_STORE_F32) {
-      C[(size_t)m * ldc + n0] = acc0[r] + (bias ? to_f32<T>(bias[n0]) : 0.f);
-      if (has1) C[(size_t)m * ldc + n0 + 1] = acc1[r] + (bias ? to_f32<T>(bias[n0 + 1]) : 0.f);
-    } else if (EPI == EPI_RESIDUAL) {
-      C[(size_t)m * ldc + n0] += acc0[r];
-      if (has1) C[(size_t)m * ldc + n0 + 1] += acc1[r];
-    } else {  // EPI_SWIGLU: row 2j = gate_j, row 2j+1 = up_j
-      float g = acc0[r], u = acc1[r];
-      C[(size_t)m * ldc + (n0 >> 1)] = g / (1.f + expf(-g)) * u;
-    }
+  if (!mine) return;
+  if (EPI == EPI_STORE_F32) {
+    C[at] = v0 + b0;
+    if (has1) C[at + 1] = v1 + b1;
+  } else if (EPI == EPI_RESIDUAL) {
+    C[at] = c0 + v0;
+    if (has1) C[at + 1] = c1 + v1;
+  } else {  // EPI_SWIGLU: row 2j = gate_j, row 2j+1 = up_j
+    C[(size_t)(m0 + lane) * ldc + (n0 >> 1)] = v0 / (1.f + expf(-v0)) * v1;
   }
 }
 
