@@ -339,8 +339,10 @@ tc_attn_merge_kernel(const float* __restrict__ part, const int32_t* __restrict__
   }
   const int total = min(len[b] + last, cap), ns = (total + keys_per_split - 1) / keys_per_split;
   const float* src = part + (size_t)pair * nsplit * (HD + 2);
-  float m_tot = -CUDART_INF_F;
-  for (int s0 = 0; s0 < ns; s0 += 32)
+  const float2 ml0 = lane < ns ? __ldcg(reinterpret_cast<const float2*>(src + (size_t)lane * (HD + 2) + HD))
+                               : make_float2(-CUDART_INF_F, 0.f);  // read once: a trip to L2 is a quarter of this kernel
+  float m_tot = ml0.x;
+  for (int s0 = 32; s0 < ns; s0 += 32)
     if (s0 + lane < ns) m_tot = fmaxf(m_tot, __ldcg(src + (size_t)(s0 + lane) * (HD + 2) + HD));
   m_tot = warp_max(m_tot);
   float denom = 0.f;
@@ -350,7 +352,7 @@ tc_attn_merge_kernel(const float* __restrict__ part, const int32_t* __restrict__
   for (int s0 = 0; s0 < ns; s0 += 32) {
     float e = 0.f, l = 0.f;  // weight and sum of split s0 + lane
     if (s0 + lane < ns) {
-      const float2 ml = __ldcg(reinterpret_cast<const float2*>(src + (size_t)(s0 + lane) * (HD + 2) + HD));
+      const float2 ml = s0 == 0 ? ml0 : __ldcg(reinterpret_cast<const float2*>(src + (size_t)(s0 + lane) * (HD + 2) + HD));
       e = ml.x == -CUDART_INF_F ? 0.f : __expf(ml.x - m_tot);
       l = ml.y;
     }
