@@ -64,8 +64,8 @@ struct ArenaPlan {
       f_gains;
   // weights packed for the tensor-core projections of batched forwards (bf16 models only)
   bool tc;
-  std::vector<LayerOff> tc_layers, ch_layers;  // w_qkv, w_o, w_gu, w_d used
-  size_t tc_head, ch_head;
+  std::vector<LayerOff> tc_layers;  // w_qkv, w_o, w_gu, w_d used
+  size_t tc_head;
 };
 
 // CTAs of the persistent kernel: one per SM of the current device (148 when none is present, the
@@ -86,19 +86,24 @@ ArenaPlan plan_arena(const ssd_model_config& c, const FastPlan* fp = nullptr) {
   size_t d = c.d_model, qd = (size_t)c.n_q_heads * c.head_dim, kvd = (size_t)c.n_kv_heads * c.head_dim;
   size_t F = c.d_ffn;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes); return o; };
+  // bf16: the row-major matrices that are uploaded become groups of 8 rows in place (chain_pack_weights)
+  auto matrix = [&](size_t rows, size_t K) {
+    const size_t b = rows * K * el;
+    return take(c.weight_dtype == 1 ? std::max(b, chain_weight_bytes((int)rows, (int)K)) : b);
+  };
   p.embed = take((size_t)(c.vocab_out + c.vocab_text) * d * el);
   p.layers.resize(c.n_layers);
   for (auto& L : p.layers) {
     L.norm1 = take(d * el);
-    L.w_qkv = take((qd + 2 * kvd) * d * el);
+    L.w_qkv = matrix(qd + 2 * kvd, d);
     L.b_qkv = take((qd + 2 * kvd) * el);
-    L.w_o = take(d * qd * el);
+    L.w_o = matrix(d, qd);
     L.norm2 = take(d * el);
-    L.w_gu = take(2 * F * d * el);
-    L.w_d = take(d * F * el);
+    L.w_gu = matrix(2 * F, d);
+    L.w_d = matrix(d, F);
   }
   p.norm_f = take(d * el);
-  p.head = take((size_t)c.vocab_out * d * el);
+  p.head = matrix((size_t)c.vocab_out, d);
   p.inv_freq = take((size_t)(c.head_dim / 2) * sizeof(double));
   p.fast = fast_supported(c);
   if (p.fast) {
@@ -128,18 +133,12 @@ ArenaPlan plan_arena(const ssd_model_config& c, const FastPlan* fp = nullptr) {
       L.w_d = take(tc_weight_bytes((int)d, (int)F));
     }
     p.tc_head = take(tc_weight_bytes(c.vocab_out, (int)d));
-    p.ch_layers.resize(c.n_layers);
-    for (auto& L : p.ch_layers) {
-      L.w_qkv = take(chain_weight_bytes((int)(qd + 2 * kvd), (int)d));
-      L.w_o = take(chain_weight_bytes((int)d, (int)qd));
-      L.w_gu = take(chain_weight_bytes((int)(2 * F), (int)d));
-      L.w_d = take(chain_weight_bytes((int)d, (int)F));
-    }
-    p.ch_head = take(chain_weight_bytes(c.vocab_out, (int)d));
   }
   p.total = off;
   return p;
 }
+
+int hd_log2_of(int head_dim) { return head_dim == 32 ? 5 : head_dim == 64 ? 6 : 7; }
 
 size_t blob_elems(const ssd_model_config& c) {
   size_t d = c.d_model, qd = (size_t)c.n_q_heads * c.head_dim, kvd = (size_t)c.n_kv_heads * c.head_dim;
@@ -421,7 +420,7 @@ int forward_chain(const ssd_model* m, ssd_streams* s, RowMap rm, const int32_t* 
   g.cap = s->cap;
   g.Hq = c.n_q_heads;
   g.Hkv = c.n_kv_heads;
-  g.hd_log2 = hd == 32 ? 5 : hd == 64 ? 6 : 7;
+  g.hd_log2 = hd_log2_of(hd);
   g.max_pages = s->max_pages;
   g.page_table = s->page_table;
   g.qscale = 1.0f / sqrtf((float)hd);
@@ -569,8 +568,9 @@ int forward(const ssd_model* m, ssd_streams* s, RowMap rm, const int32_t* draft_
   for (int l = 0; l < c.n_layers; ++l) {
     const LayerW& w = m->layers[l];
     void* kv_layer = s->kv + (size_t)l * s->kv_layer_elems * s->el;
-    SSD_CUDA(launch_gemm_simt(dt, EPI_STORE_F32, normed(w.norm1), w.w_qkv, w.b_qkv, s->qkv, qd + 2 * kvd, M,
-                              qd + 2 * kvd, d, st));
+    SimtSrc in = normed(w.norm1);
+    in.w_hd_log2 = hd_log2_of(hd);
+    SSD_CUDA(launch_gemm_simt(dt, EPI_STORE_F32, in, w.w_qkv, w.b_qkv, s->qkv, qd + 2 * kvd, M, qd + 2 * kvd, d, st));
     SSD_CUDA(launch_attention_simt(dt, s->qkv, s->rope_cs, kv_layer, s->len, rm, s->cap, c.n_q_heads, c.n_kv_heads, hd,
                                    s->part, s->nsplit_max, s->status, st));
     if (!merge_in_o)
@@ -822,36 +822,33 @@ int ssd_model_create(const ssd_model_config* cfg, const void* host_weights, size
     f.enabled = f.max_units <= FAST_MAX_UNITS && fplan.max_chunks <= FAST_MAX_CHUNKS;
   }
   if (p.tc && e == cudaSuccess) {
-    // third arrangement of the projection weights: 128-row tiles in the tensor cores' canonical
-    // shared-memory layout, made on the device from the row-major copy
+    // The matrices' other two arrangements: groups of 8 rows, in place of the rows uploaded above (tc_chain.cu and the
+    // generic kernels), and 128-row tiles in the tensor cores' canonical shared-memory layout, made from
+    // those.  The tiles' place holds the groups in between.
     ssd_tc_model& t = m->tc;
     t.n_sm = fast_cta_count();
     t.layers.resize(c.n_layers);
-    auto pack = [&](const void* src, int rows, int K, size_t dst_off) {
-      if (e == cudaSuccess) e = tc_pack_weights((const bf16*)src, rows, K, (uint8_t*)(A + dst_off), 0);
-      return (const uint8_t*)(A + dst_off);
-    };
-    // and a fourth, in groups of 8 rows that a slab of any height can be cut from (tc_chain.cu)
-    auto pack_groups = [&](const void* src, int rows, int K, size_t dst_off, int hd_log2 = 0) {
-      if (e == cudaSuccess) e = chain_pack_weights((const bf16*)src, rows, K, hd_log2, (uint8_t*)(A + dst_off), 0);
-      return (const uint8_t*)(A + dst_off);
+    auto arrange = [&](const void* rows_in_arena, int rows, int K, size_t dst_off, int hd_log2 = 0) {
+      uint8_t *groups = (uint8_t*)const_cast<void*>(rows_in_arena), *tiles = (uint8_t*)(A + dst_off);
+      if (e == cudaSuccess) e = chain_pack_weights((const bf16*)groups, rows, K, hd_log2, tiles, 0);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(groups, tiles, chain_weight_bytes(rows, K), cudaMemcpyDeviceToDevice, 0);
+      if (e == cudaSuccess) e = tc_pack_groups(groups, rows, K, hd_log2, tiles, 0);
+      return (const uint8_t*)tiles;
     };
     for (int l = 0; l < c.n_layers; ++l) {
       const LayerW& w = m->layers[l];
       const LayerOff& o = p.tc_layers[l];
-      t.layers[l].w_qkv = pack(w.w_qkv, (int)(qd + 2 * kvd), (int)d, o.w_qkv);
-      t.layers[l].w_o = pack(w.w_o, (int)d, (int)qd, o.w_o);
-      t.layers[l].w_gu = pack(w.w_gu, (int)(2 * F), (int)d, o.w_gu);
-      t.layers[l].w_d = pack(w.w_d, (int)d, (int)F, o.w_d);
-      const LayerOff& co = p.ch_layers[l];
-      t.layers[l].c_qkv = pack_groups(w.w_qkv, (int)(qd + 2 * kvd), (int)d, co.w_qkv,
-                                      c.head_dim == 32 ? 5 : c.head_dim == 64 ? 6 : 7);
-      t.layers[l].c_o = pack_groups(w.w_o, (int)d, (int)qd, co.w_o);
-      t.layers[l].c_gu = pack_groups(w.w_gu, (int)(2 * F), (int)d, co.w_gu);
-      t.layers[l].c_d = pack_groups(w.w_d, (int)d, (int)F, co.w_d);
+      t.layers[l].w_qkv = arrange(w.w_qkv, (int)(qd + 2 * kvd), (int)d, o.w_qkv, hd_log2_of(c.head_dim));
+      t.layers[l].w_o = arrange(w.w_o, (int)d, (int)qd, o.w_o);
+      t.layers[l].w_gu = arrange(w.w_gu, (int)(2 * F), (int)d, o.w_gu);
+      t.layers[l].w_d = arrange(w.w_d, (int)d, (int)F, o.w_d);
+      t.layers[l].c_qkv = (const uint8_t*)w.w_qkv;
+      t.layers[l].c_o = (const uint8_t*)w.w_o;
+      t.layers[l].c_gu = (const uint8_t*)w.w_gu;
+      t.layers[l].c_d = (const uint8_t*)w.w_d;
     }
-    t.head = pack(m->head, c.vocab_out, (int)d, p.tc_head);
-    t.c_head = pack_groups(m->head, c.vocab_out, (int)d, p.ch_head);
+    t.head = arrange(m->head, c.vocab_out, (int)d, p.tc_head);
+    t.c_head = (const uint8_t*)m->head;
     t.enabled = e == cudaSuccess;
   }
   if (e == cudaSuccess) e = cudaDeviceSynchronize();

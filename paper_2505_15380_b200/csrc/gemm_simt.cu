@@ -61,8 +61,12 @@ gemm_simt_kernel(const SimtSrc S, const T* __restrict__ W,
   const int n0 = (blockIdx.x * NG + grp) * 2;
   const bool active = n0 < N;
   const bool has1 = n0 + 1 < N;
-  const T* w0 = W + (size_t)(active ? n0 : 0) * K;
-  const T* w1 = W + (size_t)(has1 ? n0 + 1 : (active ? n0 : 0)) * K;
+  // bf16 weights lie in groups of 8 rows: a lane's 16 bytes of two neighbouring rows are one sector
+  constexpr bool GROUPS = sizeof(T) == 2;
+  constexpr int STEP = GROUPS ? 64 : 8;  // elements from 8 columns of a row to the next 8
+  const int r0 = active ? n0 : 0, r1 = has1 ? n0 + 1 : r0, steps = (K + 15) / 16;
+  const T* w0 = W + (GROUPS ? chain_elem(r0, 0, steps, S.w_hd_log2) : (size_t)r0 * K);
+  const T* w1 = W + (GROUPS ? chain_elem(r1, 0, steps, S.w_hd_log2) : (size_t)r1 * K);
   const int kc_max = K < GEMM_KC ? K : GEMM_KC;
   float acc0[GEMM_MT], acc1[GEMM_MT];
 #pragma unroll
@@ -71,10 +75,11 @@ gemm_simt_kernel(const SimtSrc S, const T* __restrict__ W,
   float x0[8], x1[8], y0[8], y1[8];
   auto load_weights = [&](int k0, int c, int nch) {
     const int c2 = c + 32 * KS < nch ? c + 32 * KS : c;
-    load8_stream(w0 + k0 + c * 8, x0);
-    load8_stream(w1 + k0 + c * 8, x1);
-    load8_stream(w0 + k0 + c2 * 8, y0);
-    load8_stream(w1 + k0 + c2 * 8, y1);
+    const size_t at = (size_t)(k0 / 8 + c) * STEP, at2 = (size_t)(k0 / 8 + c2) * STEP;
+    load8_stream(w0 + at, x0);
+    load8_stream(w1 + at, x1);
+    load8_stream(w0 + at2, y0);
+    load8_stream(w1 + at2, y1);
   };
   const int c_first = lane + 32 * ks;
   if (active && c_first < kc_max >> 3) load_weights(0, c_first, kc_max >> 3);

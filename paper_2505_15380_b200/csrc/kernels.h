@@ -49,6 +49,7 @@ struct SimtSrc {
   const int32_t* len = nullptr;
   RowMap rm{};
   int cap = 0, Hq = 0, hd = 0, nsplit_max = 0;
+  int w_hd_log2 = 0;  // bf16 W: groups of 8 rows (chain_elem), this its hd_log2.  fp32 W is row-major
 };
 cudaError_t launch_gemm_simt(int dtype, int epi, const SimtSrc& src, const void* W, const void* bias, float* C, int ldc,
                              int M, int N, int K, cudaStream_t st);

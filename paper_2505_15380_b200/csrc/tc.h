@@ -232,6 +232,8 @@ cudaError_t launch_tc_prefill_gemm(const TcGemm& g, int epi, const bf16* bias, f
 
 // tc_gemm.cu
 cudaError_t tc_pack_weights(const bf16* w_rowmajor, int n_rows, int K, uint8_t* packed, cudaStream_t st);
+// The same from groups of 8 rows (chain_pack_weights).
+cudaError_t tc_pack_groups(const uint8_t* groups, int n_rows, int K, int hd_log2, uint8_t* packed, cudaStream_t st);
 cudaError_t tc_unpack_weights(const uint8_t* packed, int n_rows, int K, bf16* w_rowmajor, cudaStream_t st);
 cudaError_t launch_tc_gemm(const TcGemm& g, cudaStream_t st);
 
@@ -270,7 +272,15 @@ struct ChainSplit {
 };
 inline bool chain_long(int K) { return K > 2048; }
 inline size_t chain_weight_bytes(int n_rows, int K) { return (size_t)((n_rows + 7) / 8) * ((K + 15) / 16) * 256; }
-// hd_log2: rows of the QKV projection, whose rotary partners become neighbours; 0: any other.
+// Element of such a copy at which 8 columns c8 * 8 .. of a weight row begin (the next 8 are 64 elements on).
+// hd_log2: rows of the QKV projection, whose rotary partners are neighbours; 0: any other.
+__host__ __device__ inline size_t chain_elem(int row, int c8, int KS, int hd_log2) {
+  if (hd_log2) {
+    const int j = row & ((1 << hd_log2) - 1), half = 1 << (hd_log2 - 1);
+    row += ((j & (half - 1)) << 1) + (j >> (hd_log2 - 1)) - j;
+  }
+  return ((size_t)(row >> 3) * KS * 2 + c8) * 64 + (size_t)(row & 7) * 8;
+}
 cudaError_t chain_pack_weights(const bf16* w_rowmajor, int n_rows, int K, int hd_log2, uint8_t* packed, cudaStream_t st);
 // whole: a projection whose CTAs take all token rows whatever their number (gate/up and down).  Its operand
 // is arranged in the chunks of rows that its CTAs take.

@@ -385,8 +385,9 @@ __global__ void __launch_bounds__(TC_THREADS) tc_gemm_kernel(const __grid_consta
 
 // ---- weight packing (once per model) -----------------------------------------------------------
 
-__global__ void tc_pack_weights_kernel(const bf16* __restrict__ w, int n_rows, int K, int KS, size_t n_chunks,
-                                       uint4* __restrict__ out) {
+template <bool GROUPS>
+__global__ void tc_pack_weights_kernel(const bf16* __restrict__ w, int n_rows, int K, int KS, int hd_log2,
+                                       size_t n_chunks, uint4* __restrict__ out) {
   // one thread = one 16-byte row of a core matrix: chunk = ((tile * KS + ks) * 2 + kc) * 128 + r
   const size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= n_chunks) return;
@@ -395,7 +396,8 @@ __global__ void tc_pack_weights_kernel(const bf16* __restrict__ w, int n_rows, i
   const int ks = (int)(blk % KS), tile = (int)(blk / KS);
   const int n = tile * TC_TILE_ROWS + r, k0 = ks * 16 + kc * 8;
   uint4 v = make_uint4(0u, 0u, 0u, 0u);
-  if (n < n_rows && k0 < K) v = *reinterpret_cast<const uint4*>(w + (size_t)n * K + k0);  // K is a multiple of 8
+  if (n < n_rows && k0 < K)  // K is a multiple of 8
+    v = *reinterpret_cast<const uint4*>(w + (GROUPS ? chain_elem(n, k0 >> 3, KS, hd_log2) : (size_t)n * K + k0));
   out[c] = v;
 }
 
@@ -415,8 +417,17 @@ __global__ void tc_unpack_weights_kernel(const uint4* __restrict__ packed, int n
 cudaError_t tc_pack_weights(const bf16* w, int n_rows, int K, uint8_t* packed, cudaStream_t st) {
   const int KS = (K + 15) / 16;
   const size_t n_chunks = tc_weight_bytes(n_rows, K) / 16;
-  tc_pack_weights_kernel<<<(unsigned)((n_chunks + 255) / 256), 256, 0, st>>>(w, n_rows, K, KS, n_chunks,
-                                                                            reinterpret_cast<uint4*>(packed));
+  tc_pack_weights_kernel<false><<<(unsigned)((n_chunks + 255) / 256), 256, 0, st>>>(w, n_rows, K, KS, 0, n_chunks,
+                                                                                   reinterpret_cast<uint4*>(packed));
+  count_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t tc_pack_groups(const uint8_t* groups, int n_rows, int K, int hd_log2, uint8_t* packed, cudaStream_t st) {
+  const int KS = (K + 15) / 16;
+  const size_t n_chunks = tc_weight_bytes(n_rows, K) / 16;
+  tc_pack_weights_kernel<true><<<(unsigned)((n_chunks + 255) / 256), 256, 0, st>>>(
+      reinterpret_cast<const bf16*>(groups), n_rows, K, KS, hd_log2, n_chunks, reinterpret_cast<uint4*>(packed));
   count_launch();
   return cudaGetLastError();
 }
